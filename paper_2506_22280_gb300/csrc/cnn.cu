@@ -32,6 +32,7 @@ constexpr int kFeat = 8 * 8 * 128;
 constexpr int kFeatIn = kFeat + 2;
 constexpr int kHid = 128;
 constexpr int kMaxBatch = 1024;
+constexpr int kFc2Blocks = 16;  // blocks of the output layer's weight gradient
 
 struct ParamOffsets {
   size_t w[kConvs], b[kConvs], w1, b1, w2, b2, total;
@@ -63,18 +64,11 @@ size_t kdim(int l) { return (size_t)9 * kCh[l]; }
 
 // Workspace of one batch: activations for the backward, gradients, split-K partials, BF16 copies.
 struct CnnWs {
-  float *col[kConvs], *act[kConvs], *feat, *h, *out, *dout, *dh, *dfeat, *dact0, *dact1, *dcol, *part, *loss;
+  float *h, *out, *dout, *dh, *part, *loss;
+  CnnF32 f32;  // the FP32 path's activations, gradients and partial sums (cnn_f32.cu)
   CnnTc tc;  // the tensor-core path's BF16 activations, gradients and weight copies (cnn_tc.cu)
   size_t bytes;
 };
-
-constexpr int kSplits = 32;
-
-// Floats of the split-K partial buffer: 32 splits of the largest dW (128 x 1152) or 16 splits of the
-// B x 128 hidden layer, whichever is more.
-long long part_floats(int B) {
-  return std::max<long long>((long long)kSplits * 128 * 1152, 16LL * B * 128);
-}
 
 CnnWs cnn_layout(void* base, int B, int R) {
   CnnWs w;
@@ -85,119 +79,16 @@ CnnWs cnn_layout(void* base, int B, int R) {
     off += (bytes + 255) & ~(size_t)255;
     return q;
   };
-  size_t max_act = 0, max_col = 0;
-  for (int l = 0; l < kConvs; ++l) {
-    w.col[l] = (float*)take(rows(l, B) * kdim(l) * 4);
-    w.act[l] = (float*)take(rows(l, B) * kCh[l + 1] * 4);
-    max_act = std::max(max_act, rows(l, B) * kCh[l + 1]);
-    max_col = std::max(max_col, rows(l, B) * kdim(l));
-  }
-  max_act = std::max(max_act, (size_t)B * kFeatIn);
-  w.feat = (float*)take((size_t)B * kFeatIn * 4);
   w.h = (float*)take((size_t)B * kHid * 4);
   w.out = (float*)take((size_t)B * R * 4 + 4);
   w.dout = (float*)take((size_t)B * R * 4 + 4);
   w.dh = (float*)take((size_t)B * kHid * 4);
-  w.dfeat = (float*)take((size_t)B * kFeatIn * 4);
-  w.dact0 = (float*)take(max_act * 4);
-  w.dact1 = (float*)take(max_act * 4);
-  w.dcol = (float*)take(max_col * 4);
-  w.part = (float*)take((size_t)part_floats(B) * 4);  // split-K and bias partials
+  w.part = (float*)take((size_t)kFc2Blocks * R * (kHid + 1) * 4);  // output-layer weight-gradient partials
   w.loss = (float*)take(256);
+  off += cnn_f32_layout(p ? p + off : nullptr, B, &w.f32);
   off += cnn_tc_layout(p ? p + off : nullptr, B, &w.tc);
   w.bytes = off;
   return w;
-}
-
-__device__ __forceinline__ float to_f(float x) { return x; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
-template <typename T>
-__device__ __forceinline__ T from_f(float x);
-template <>
-__device__ __forceinline__ float from_f<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
-// C(m, n) = sum_k A(m, k) B(k, n) over this block's k-range; A(m, k) = AT ? A[k lda + m] : A[m lda + k],
-// B(k, n) = BT ? B[n ldb + k] : B[k ldb + n].  64 x 64 tile per 256 threads (4 x 4 per thread), 16-deep
-// k slices in shared memory.  gridDim.z > 1: block z sums k in [z kchunk, (z + 1) kchunk) and writes its
-// partial to C + z * zstride (summed later); else the epilogue adds bias[n] and applies ReLU if asked.
-template <bool AT, bool BT, typename TA, typename TB, typename TC>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const TA* __restrict__ A, int lda,
-                                              const TB* __restrict__ B, int ldb, TC* __restrict__ C, int ldc,
-                                              int kchunk, long long zstride, const float* __restrict__ bias,
-                                              int relu) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int k0 = kb; k0 < ke; k0 += 16) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int t = threadIdx.x + 256 * e;  // 1024 elements of each 64 x 16 slice
-      int mm, kk;
-      if (AT) { kk = t >> 6; mm = t & 63; } else { mm = t >> 4; kk = t & 15; }
-      const int m = m0 + mm, k = k0 + kk;
-      float a = 0.f;
-      if (m < M && k < ke) a = to_f(AT ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k]);
-      As[kk][mm] = a;
-      int nn, kk2;
-      if (BT) { nn = t >> 4; kk2 = t & 15; } else { kk2 = t >> 6; nn = t & 63; }
-      const int n = n0 + nn, k2 = k0 + kk2;
-      float bv = 0.f;
-      if (n < N && k2 < ke) bv = to_f(BT ? B[(size_t)n * ldb + k2] : B[(size_t)k2 * ldb + n]);
-      Bs[kk2][nn] = bv;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  TC* Cz = C + (size_t)blockIdx.z * zstride;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      float v = acc[i][j];
-      if (gridDim.z == 1) {
-        if (bias) v += bias[n];
-        if (relu) v = fmaxf(v, 0.f);
-      }
-      Cz[(size_t)m * ldc + n] = from_f<TC>(v);
-    }
-  }
-}
-
-template <bool AT, bool BT, typename TA, typename TB, typename TC>
-cudaError_t gemm(int M, int N, int K, const TA* A, int lda, const TB* B, int ldb, TC* C, int ldc, const float* bias,
-                 bool relu, cudaStream_t st, int splits = 1, long long zstride = 0) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  const int kchunk = ((K + splits - 1) / splits + 15) / 16 * 16;
-  dim3 grid((N + 63) / 64, (M + 63) / 64, splits);
-  k_gemm<AT, BT, TA, TB, TC><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, kchunk, zstride, bias,
-                                                   relu ? 1 : 0);
-  note_launches(1);
-  return cudaGetLastError();
 }
 
 // The R-wide output layer, FP32: out[b][r] = b2[r] + sum_n h[b][n] W2[r][n], one warp per batch entry.
@@ -265,104 +156,7 @@ __global__ void k_sum_splits(const float* __restrict__ part, int splits, long lo
   out[i] = s;
 }
 
-// db[n] = sum_m dY[m][n]: each block sums 32 columns over a slice of rows (lane = column), then the
-// slices are summed in order.
-__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ dY, int M, int N, int rows_per,
-                                                float* __restrict__ part) {
-  __shared__ float red[8][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n = blockIdx.x * 32 + lane;
-  const int m0 = blockIdx.y * rows_per, m1 = min(M, m0 + rows_per);
-  float s = 0.f;
-  if (n < N)
-    for (int m = m0 + warp; m < m1; m += 8) s += dY[(size_t)m * N + n];
-  red[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0 && n < N) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
-    part[(size_t)blockIdx.y * N + n] = t;
-  }
-}
-
-cudaError_t colsum(const float* dY, int M, int N, float* part, float* db, cudaStream_t st) {
-  // about 4096 rows per slice (at least kSplits slices), so that tall thin dY fill the GPU
-  const int splits = std::max(kSplits, std::min((M + 4095) / 4096, 1024));
-  const int rows_per = (M + splits - 1) / splits;
-  dim3 grid((N + 31) / 32, splits);
-  k_colsum<<<grid, 256, 0, st>>>(dY, M, N, rows_per, part);
-  k_sum_splits<<<(N + 255) / 256, 256, 0, st>>>(part, splits, N, db, 0);
-  note_launches(2);
-  return cudaGetLastError();
-}
-
-// col[(b Ho + y) Wo + x][(ky 3 + kx) C + c] = in[b][2y + ky - 1][2x + kx - 1][c] (0 outside), NHWC.
-template <typename TI, typename TO>
-__global__ void k_im2col(const TI* __restrict__ in, int B, int H, int W, int C, TO* __restrict__ col) {
-  const int Ho = H / 2, Wo = W / 2, K = 9 * C;
-  const long long total = (long long)B * Ho * Wo * K;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int k = (int)(i % K);
-    const long long r = i / K;
-    const int x = (int)(r % Wo), y = (int)((r / Wo) % Ho), b = (int)(r / ((long long)Wo * Ho));
-    const int c = k % C, tap = k / C, ky = tap / 3, kx = tap % 3;
-    const int iy = 2 * y + ky - 1, ix = 2 * x + kx - 1;
-    float v = 0.f;
-    if (iy >= 0 && iy < H && ix >= 0 && ix < W) v = to_f(in[(((size_t)b * H + iy) * W + ix) * C + c]);
-    col[i] = from_f<TO>(v);
-  }
-}
-
-// din[b][iy][ix][c] = sum over the taps that read it of dcol[(b Ho + y) Wo + x][(ky 3 + kx) C + c].
-__global__ void k_col2im(const float* __restrict__ dcol, int B, int H, int W, int C, float* __restrict__ din) {
-  const int Ho = H / 2, Wo = W / 2, K = 9 * C;
-  const long long total = (long long)B * H * W * C;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long r = i / C;
-    const int ix = (int)(r % W), iy = (int)((r / W) % H), b = (int)(r / ((long long)W * H));
-    float s = 0.f;
-#pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-      const int ty = iy + 1 - ky;
-      if (ty < 0 || (ty & 1) || (ty >> 1) >= Ho) continue;
-#pragma unroll
-      for (int kx = 0; kx < 3; ++kx) {
-        const int tx = ix + 1 - kx;
-        if (tx < 0 || (tx & 1) || (tx >> 1) >= Wo) continue;
-        s += dcol[(((size_t)b * Ho + (ty >> 1)) * Wo + (tx >> 1)) * K + (ky * 3 + kx) * C + c];
-      }
-    }
-    din[i] = s;
-  }
-}
-
 unsigned grid_for(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 152LL * 32); }
-
-// feat[b] = (act3[b] (8192 values), cos theta_b, sin theta_b)
-template <typename TI, typename TO>
-__global__ void k_features(const TI* __restrict__ act3, const float* __restrict__ cs, int B, TO* __restrict__ feat) {
-  const long long total = (long long)B * kFeatIn;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(i / kFeatIn), j = (int)(i % kFeatIn);
-    const float v = j < kFeat ? to_f(act3[(size_t)b * kFeat + j]) : cs[2 * b + (j - kFeat)];
-    feat[i] = from_f<TO>(v);
-  }
-}
-
-// dact3[b][j] = dfeat[b][j] for the image features (the angle inputs get no gradient).
-__global__ void k_feat_grad(const float* __restrict__ dfeat, int B, float* __restrict__ dact3) {
-  const long long total = (long long)B * kFeat;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-    dact3[i] = dfeat[(i / kFeat) * kFeatIn + i % kFeat];
-}
-
-// dY *= [Y > 0] (ReLU backward; Y is the post-activation value).
-__global__ void k_relu_bwd(const float* __restrict__ Y, long long n, float* __restrict__ dY) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    if (!(Y[i] > 0.f)) dY[i] = 0.f;
-}
 
 // loss = mean (out - target)^2 over B x R; dout = 2 (out - target) / (B R).  One block.
 __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ out, const float* __restrict__ target, int n,
@@ -395,11 +189,6 @@ __global__ void k_downsample(const float* __restrict__ proj, int B, int nu, int 
     const float* p = proj + ((size_t)b * nv + f * y) * nu + f * x;
     img[i] = f == 2 ? 0.25f * scale * (p[0] + p[1] + p[nu] + p[nu + 1]) : scale * p[0];
   }
-}
-
-__global__ void k_to_bf16(const float* __restrict__ x, long long n, __nv_bfloat16* __restrict__ y) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16_rn(x[i]);
 }
 
 // He-normal weights (std sqrt(2 / fan_in)) from a counter-based generator (splitmix64 of seed and index,
@@ -466,19 +255,7 @@ cudaError_t forward_f32(const NetPtrs<float>& N, int R, const float* img, const 
   if (tc) {
     CNN_TRY(cnn_tc_forward(cnn_net(N), img, cs, B, w.tc, w.h, st));
   } else {
-    const float* in = img;
-    for (int l = 0; l < kConvs; ++l) {
-      const int H = kEdge[l], C = kCh[l];
-      const long long ncol = (long long)rows(l, B) * kdim(l);
-      k_im2col<float, float><<<grid_for(ncol), 256, 0, st>>>(in, B, H, H, C, w.col[l]);
-      note_launches(1);
-      CNN_TRY(gemm<false, true>((int)rows(l, B), kCh[l + 1], (int)kdim(l), w.col[l], (int)kdim(l), N.w[l],
-                                (int)kdim(l), w.act[l], kCh[l + 1], N.b[l], true, st));
-      in = w.act[l];
-    }
-    k_features<float, float><<<grid_for((long long)B * kFeatIn), 256, 0, st>>>(w.act[kConvs - 1], cs, B, w.feat);
-    note_launches(1);
-    CNN_TRY(gemm<false, true>(B, kHid, kFeatIn, w.feat, kFeatIn, N.w1, kFeatIn, w.h, kHid, N.b1, true, st));
+    CNN_TRY(cnn_f32_forward(cnn_net(N), img, cs, B, w.f32, w.h, st));
   }
   k_fc2_fwd<<<(B + 7) / 8, 256, 0, st>>>(w.h, N.w2, N.b2, B, R, w.out);
   note_launches(1);
@@ -489,50 +266,18 @@ cudaError_t forward_f32(const NetPtrs<float>& N, int R, const float* img, const 
 cudaError_t backward_f32(const NetPtrs<float>& N, const ParamOffsets& o, int R, int B, const CnnWs& w, float* grad,
                          bool tc, cudaStream_t st) {
   // output layer
-  constexpr int kFc2Blocks = 16;
   k_fc2_wgrad<<<kFc2Blocks, kHid + 32, 0, st>>>(w.dout, w.h, B, R, w.part);
   k_sum_splits<<<(R * kHid + R + 255) / 256, 256, 0, st>>>(w.part, kFc2Blocks, R * kHid + R, grad + o.w2, 0);
   k_fc2_dh<<<(B * kHid + 255) / 256, 256, 0, st>>>(w.dout, N.w2, w.h, B, R, w.dh, tc ? w.tc.dhb : nullptr);
   note_launches(3);
-  CNN_TRY(colsum(w.dh, B, kHid, w.part, grad + o.b1, st));
-  if (tc) {
-    CnnGrad g;
-    for (int l = 0; l < kConvs; ++l) {
-      g.w[l] = grad + o.w[l];
-      g.b[l] = grad + o.b[l];
-    }
-    g.w1 = grad + o.w1;
-    return cnn_tc_backward(B, w.tc, w.dh, g, st);
+  CNN_TRY(cnn_colsum(w.dh, B, kHid, w.tc, grad + o.b1, st));
+  CnnGrad g;
+  for (int l = 0; l < kConvs; ++l) {
+    g.w[l] = grad + o.w[l];
+    g.b[l] = grad + o.b[l];
   }
-  // hidden layer
-  CNN_TRY(gemm<true, false>(kHid, kFeatIn, B, w.dh, kHid, w.feat, kFeatIn, grad + o.w1, kFeatIn, nullptr, false, st));
-  CNN_TRY(gemm<false, false>(B, kFeatIn, kHid, w.dh, kHid, N.w1, kFeatIn, w.dfeat, kFeatIn, nullptr, false, st));
-  k_feat_grad<<<grid_for((long long)B * kFeat), 256, 0, st>>>(w.dfeat, B, w.dact0);
-  note_launches(1);
-  // convolutions, last to first; dact0 holds dL/d(output of conv l)
-  float* dY = w.dact0;
-  float* dX = w.dact1;
-  for (int l = kConvs - 1; l >= 0; --l) {
-    const int M = (int)rows(l, B), Nn = kCh[l + 1], K = (int)kdim(l);
-    k_relu_bwd<<<grid_for((long long)M * Nn), 256, 0, st>>>(w.act[l], (long long)M * Nn, dY);
-    note_launches(1);
-    const long long ndw = (long long)Nn * K;
-    const int splits = kSplits;  // split the B x H x W rows: dW is at most 128 x 1152
-    CNN_TRY(gemm<true, false>(Nn, K, M, dY, Nn, w.col[l], K, w.part, K, nullptr, false, st, splits, ndw));
-    k_sum_splits<<<(unsigned)((ndw + 255) / 256), 256, 0, st>>>(w.part, splits, ndw, grad + o.w[l], 0);
-    note_launches(1);
-    CNN_TRY(colsum(dY, M, Nn, w.part, grad + o.b[l], st));
-    if (l > 0) {
-      CNN_TRY(gemm<false, false>(M, K, Nn, dY, Nn, N.w[l], K, w.dcol, K, nullptr, false, st));
-      const int H = kEdge[l], C = kCh[l];
-      k_col2im<<<grid_for((long long)B * H * H * C), 256, 0, st>>>(w.dcol, B, H, H, C, dX);
-      note_launches(1);
-      float* t = dY;
-      dY = dX;
-      dX = t;
-    }
-  }
-  return cudaGetLastError();
+  g.w1 = grad + o.w1;
+  return tc ? cnn_tc_backward(B, w.tc, w.dh, g, st) : cnn_f32_backward(cnn_net(N), B, w.f32, w.tc, w.dh, g, st);
 }
 
 bool args_ok(int R, int B) { return R >= 1 && R <= DIGS_MAX_R && B >= 1 && B <= kMaxBatch; }

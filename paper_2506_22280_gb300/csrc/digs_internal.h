@@ -157,6 +157,25 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
 // t.dhb, written by the caller with it), through the activations and weights that the last
 // cnn_tc_forward on the same buffers kept.
 cudaError_t cnn_tc_backward(int B, const CnnTc& t, const float* dh, const CnnGrad& g, cudaStream_t st);
+// out[c] = sum over the M rows of dY [M][N] (FP32), in a fixed order (t: scratch).
+cudaError_t cnn_colsum(const float* dY, int M, int N, const CnnTc& t, float* out, cudaStream_t st);
+// For the FP32 mode: the first convolution's weight gradient [32][9] from dY [B 4096][32] and the images
+// (t: scratch), and out[i] = sum over z of part[z n + i] (+ bias[i % nb] and ReLU when bias is given).
+cudaError_t cnn_conv0_dw_f32(const float* dy, const float* img, int B, const CnnTc& t, float* out, cudaStream_t st);
+cudaError_t cnn_sum_splits(const float* part, int Z, long long n, const float* bias, int nb, float* out, cudaStream_t st);
+
+// cnn_f32.cu: the same network in FP32 on the SIMT pipes (buffers of one batch size, all FP32).
+struct CnnF32 {
+  float *img, *act[3], *feat, *dy[2], *part;
+  long long part_floats;
+};
+size_t cnn_f32_layout(void* base, int B, CnnF32* t);
+cudaError_t cnn_f32_forward(const CnnNet& net, const float* img, const float* cs, int B, const CnnF32& t, float* h,
+                            cudaStream_t st);
+// As cnn_tc_backward, from dh through what the last cnn_f32_forward on the same buffers kept; tc: scratch of
+// the column sums.
+cudaError_t cnn_f32_backward(const CnnNet& net, int B, const CnnF32& t, const CnnTc& tc, const float* dh, const CnnGrad& g,
+                             cudaStream_t st);
 
 // adam.cu
 struct AdamGroup {
