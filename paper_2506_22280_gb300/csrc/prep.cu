@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(128, 5) k_prep_fwd(GaussPtrs g, const __grid_c
       tb = make_uint2((uint32_t)(x0 / tile) | ((uint32_t)(y0 / tile) << 16), (uint32_t)(x1 / tile) | ((uint32_t)(y1 / tile) << 16));
       cost = min(((uint32_t)(x1 - x0 + 1) * (uint32_t)(y1 - y0 + 1) + 31u) >> 5, 255u);  // backward passes
     } else {
-      r = Rec{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0, 0, 0};
+      r = Rec{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0, 0, 0.f};
     }
     size_t idx = (size_t)b * sc.nmax + n;
     store_rec(rec + idx * DIGS_REC_F4, r);

@@ -7,13 +7,16 @@
 // reciprocal square root.  Pixels are taken two at a time in packed FP32x2 arithmetic
 // (fma/mul/add.rn.f32x2).
 //
-// Forward: one CTA per (projection, tile) and one warp per 8 x 8 block of the tile; each lane owns two
-// pixels of the block and keeps their sums in registers.  Every warp walks the tile's sorted Gaussian
-// list in batches of 32 records staged by cp.async, keeps the Gaussians whose cutoff ellipse meets its
-// block and sweeps them eight at a time, summed in list order: no canvas, no atomics, deterministic sums.
-// An entry carries its quadratic form scaled by 1/|amp|^2 (and t by 1/|amp|), so that the reciprocal
-// square root of the scaled D is |amp| D^-1/2; the accumulating FMA applies the sign of amp.  CTAs start
-// in order of decreasing list length.
+// Forward: a warp owns two 8 x 8 blocks, side by side, of a (projection, tile), each lane two pixels of both with
+// their sums in registers; the warps of a CTA share its pixels and split its sorted Gaussian list.  A warp takes
+// 32 records at a time, one per lane, writes an entry for every block whose pixels the record's cutoff ellipse
+// can reach, and sweeps each block's entries, four per step, in list order: no canvas, no atomics, sums that do
+// not depend on timing.  CTAs start in order of decreasing list length.
+// What bounds it: instruction issue, about 25 instructions per entry and block of 64 pixels (FMA and SFU pipes
+// each about 60 % busy), then loading and testing the records.  One block per warp made every block load and
+// test the whole list by itself: a third of the time.  128 thorax projections (100k Gaussians, 256^2):
+// 5.31 -> 4.22 ms; 16: 0.78 -> 0.57; 8 of 500k Gaussians on 512^2: 5.2 -> 3.8; 16 of 2,000 on 64^2:
+// 0.044 -> 0.023.
 //
 // Backward: needs no tile lists.  One half-warp per (projection, Gaussian) record (the two records of a
 // warp of similar box size, paired by k_bwd_pairing) sweeps the record's pixel box in 16-column slices,
@@ -129,190 +132,238 @@ __device__ __forceinline__ HalfLanes group_lanes(int w, int h, int hl) {
 
 // ---- forward ------------------------------------------------------------------------------------
 
-// One CTA per (projection, tile), launched in the order `order` gives; one warp per 8 x 8 block of the tile.  Lane l owns the pixels
-// (l mod 8, l div 8) and (l mod 8, l div 8 + 4) of its block and keeps their sums in a register pair.
-template <int TS>
+// A CTA takes 16 x 16 pixels of a (projection, tile) (tiles of 32 pixels: four CTAs share a list), or a tile of
+// 8 x 8; tiles in the order `order` gives.  A warp owns NB of its 8 x 8 blocks and every SP-th batch of the
+// list; lane l owns the pixels (l mod 8, l div 8) and (l mod 8, l div 8 + 4) of each block and keeps their sums
+// in registers.
+template <int TS, int NB, int SP>
 struct FwdCfg {
-  static constexpr int blocks_x = TS / 8;
-  static constexpr int warps = blocks_x * blocks_x;
+  static constexpr int groups = TS == 8 ? 1 : 4 / NB;  // warps that share the CTA's blocks
+  static constexpr int warps = groups * SP;
+  static constexpr int subs = TS == 32 ? 4 : 1;        // CTAs per tile
   static constexpr int threads = 32 * warps;
-  static constexpr int batch = 32;                              // records a warp stages at a time
-  static constexpr int raw_f4 = batch * DIGS_REC_F4;            // staged records
-  static constexpr int ent_f4 = batch * 3;                      // derived entries
-  static constexpr size_t smem = (size_t)warps * (raw_f4 + ent_f4) * sizeof(float4);
+  static constexpr int batch = 32;                     // records a warp takes at a time: one per lane
+  // CTAs per SM that the registers are held to: 28 warps of 72 registers (NB = 1: 32 of 64).  For 128 thorax
+  // projections, 24, 28 and 32 warps took 4.41, 4.22 and 4.41 ms.
+  static constexpr int min_ctas = (NB == 1 ? 32 : 28) / warps;
 };
 
-// A staged record -> the entry the pixel loop reads:
-//   (k n00 / sg^2, k n01x2 / sg^2, k n11 / sg^2, wn0 / sg), (wn1 / sg, kappa / k, amp / sg, -xc), (-yc, 1 / sg, 0, 0)
-// with k = -log2(e) / 2, so that the loop forms the exp2 argument k E = k num / D directly, and
-// sg = |amp| (1 when |amp| lies outside [2^-40, 2^40]): num and t scaled by 1 / sg^2 and 1 / sg scale D
-// by 1 / sg^2 and leave E unchanged, so the SFU's rsqrt of the scaled D is sg D^-1/2 and the amplitude
-// costs no multiply in the loop (amp / sg, i.e. the sign of amp, is applied by the accumulating FMA).
-__device__ __forceinline__ void derive_entry(const float4* raw, float4* ent) {
-  const float4 a = raw[0], b = raw[1], c = raw[2];
+// A record's share of the entries that the pixel loops read, the same for every block: with k = -log2(e) / 2 and
+// sg = |amp| (1 when |amp| lies outside [2^-40, 2^40]), the quadratic form times k / sg^2, t's slopes over sg,
+// kappa / k and amp / sg.  The loop then forms the exp2 argument k E = k num / D directly; num and t scaled by
+// 1 / sg^2 and 1 / sg scale D by 1 / sg^2 and leave E unchanged, so the SFU's rsqrt of the scaled D is
+// sg D^-1/2 (amp / sg, i.e. the sign of amp, multiplies both pixels of a lane at once).
+struct FwdScaled {
+  float n00, n01, n11, t1, t2, s1, kap, sgn;
+};
+__device__ __forceinline__ FwdScaled scale_record(const float4& a, const float4& b, const float4& c) {
   const float mag = fabsf(c.x);
   const bool fold = mag >= 0x1p-40f && mag <= 0x1p40f;
-  const float s1 = fold ? __frcp_rn(mag) : 1.f, s2 = s1 * s1;
-  const float sgn = fold ? copysignf(1.f, c.x) : c.x;
-  ent[0] = make_float4(kNegHalfLog2e * a.z * s2, kNegHalfLog2e * a.w * s2, kNegHalfLog2e * b.x * s2, b.y * s1);
-  ent[1] = make_float4(b.z * s1, b.w * (1.f / kNegHalfLog2e), sgn, -a.x);
-  ent[2] = make_float4(-a.y, s1, 0.f, 0.f);
+  FwdScaled r;
+  r.s1 = fold ? __frcp_rn(mag) : 1.f;
+  r.sgn = fold ? copysignf(1.f, c.x) : c.x;
+  const float s2 = r.s1 * r.s1 * kNegHalfLog2e;
+  r.n00 = a.z * s2;
+  r.n01 = a.w * s2;
+  r.n11 = b.x * s2;
+  r.t1 = b.y * r.s1;
+  r.t2 = b.z * r.s1;
+  r.kap = b.w * (1.f / kNegHalfLog2e);
+  return r;
 }
 
-// Whether the pixel rectangle [x0, x1] x [y0, y1] (a block's part of the record's box) can hold a pixel
-// with E <= c2: E = num / D with D <= Dmax = (1 + tau)^2 / (1 - c2 kappa) over the box (|t - 1| <= tau,
-// kappa num <= c2 kappa D), so no pixel qualifies when min over the rectangle of the quadratic form num
-// exceeds c2 Dmax.  The minimum of a positive definite form over a rectangle not holding its centre lies
-// on an edge, where it is a clamped one-dimensional minimum.  Conservative (small relative margin); a
-// culled block's entries would only have added zeros, so sums are unchanged.
-__device__ __forceinline__ bool ellipse_meets(const float4* r3, int x0, int x1, int y0, int y1, float c2_const) {
-  const float4 a = r3[0], b = r3[1], c = r3[2];
-  const float xc = a.x, yc = a.y, n00 = a.z, n01 = 0.5f * a.w, n11 = b.x;
-  const float X0 = (float)x0 - xc, X1 = (float)x1 - xc, Y0 = (float)y0 - yc, Y1 = (float)y1 - yc;
-  if (X0 <= 0.f && X1 >= 0.f && Y0 <= 0.f && Y1 >= 0.f) return true;
-  const int bx = __float_as_int(c.y), by = __float_as_int(c.z);
-  const float mdx = fmaxf(fabsf((float)(bx & 0xffff) - xc), fabsf((float)(bx >> 16) - xc));
-  const float mdy = fmaxf(fabsf((float)(by & 0xffff) - yc), fabsf((float)(by >> 16) - yc));
-  const float tau = fabsf(b.y) * mdx + fabsf(b.z) * mdy;
-  const float ck = 1.f - c2_const * b.w;  // > 0: the source lies outside the cutoff ellipsoid
-  if (!(ck > 0.f)) return true;
-  // fast (approximate) divisions: they move the clamped minimisers by a few ulps, far inside the margin
-  const float lim = __fdividef(c2_const * (1.f + tau) * (1.f + tau), ck) * 1.001f + 1e-4f;
-  const float s11 = __fdividef(-n01, n11), s00 = __fdividef(-n01, n00);
-  auto q = [&](float dx, float dy) { return dy * (n11 * dy + 2.f * n01 * dx) + n00 * dx * dx; };
-  auto edge_x = [&](float dx) {  // min over dy in [Y0, Y1] at fixed dx
-    const float dy = fminf(fmaxf(s11 * dx, Y0), Y1);
-    return q(dx, dy);
-  };
-  auto edge_y = [&](float dy) {
-    const float dx = fminf(fmaxf(s00 * dy, X0), X1);
-    return q(dx, dy);
-  };
-  const float m = fminf(fminf(edge_x(X0), edge_x(X1)), fminf(edge_y(Y0), edge_y(Y1)));
-  return !(m > lim);
+// The entry of one 8 x 8 block.  With (X, Y) the block centre's offset from the projected mean and (x, y) a
+// pixel's offset from the block centre (x, y in -3.5 ... 3.5),
+//   k num / sg^2 = a0 + x (a1 + x a2) + y (b0 + x b1 + y c),  t / sg = t0 + x t1 + y t2,
+// so that x and y are constants of the lane: a column costs four FMAs and a row three, with no offset to form.
+__device__ __forceinline__ void write_entry(const FwdScaled& r, float X, float Y, float4* ent) {
+  const float h0 = r.n00 * X, h1 = r.n11 * Y;
+  ent[0] = make_float4(r.n00, r.n01, fmaf(r.n01, Y, 2.f * h0), fmaf(r.n01, X, 2.f * h1));  // a2, b1, a1, b0
+  ent[1] = make_float4(fmaf(X, fmaf(r.n01, Y, h0), h1 * Y), fmaf(r.t1, X, fmaf(r.t2, Y, r.s1)), r.t1, r.n11);  // a0, t0, t1, c
+  ent[2] = make_float4(r.t2, r.kap, r.sgn, 0.f);
 }
 
-__device__ __forceinline__ f2 f2_lo(const float4& v) { return f2_pack(v.x, v.y); }
-__device__ __forceinline__ f2 f2_hi(const float4& v) { return f2_pack(v.z, v.w); }
+// Whether the 8 x 8 pixel block whose centre lies at (X, Y) from the projected mean can hold a pixel with
+// E <= c2: E = num / D with D <= Dmax over the record's box, and lim = c2 Dmax (with a small margin, from the
+// set-up), so no pixel qualifies when min over the block of the quadratic form num exceeds lim.  The minimum
+// of a positive definite form over a rectangle lies on one of the two edges that face its centre (or on a
+// line through the centre, where the rectangle spans it), and on such a line it is a clamped one-dimensional
+// minimum; a centre inside the block gives zero.  A culled block's entries would only have added zeros.
+// sy = -n01 / n11 and sx = -n01 / n00 (n01x2 = 2 n01) from approximate divisions: they move the clamped
+// minimisers by a few ulps, far inside the margin.
+__device__ __forceinline__ bool ellipse_meets(float n00, float n01x2, float n11, float sx, float sy, float lim, float X,
+                                              float Y) {
+  const float X0 = X - 3.5f, X1 = X + 3.5f, Y0 = Y - 3.5f, Y1 = Y + 3.5f;
+  const float ex = fminf(fmaxf(0.f, X0), X1), ey = fminf(fmaxf(0.f, Y0), Y1);
+  const float dy = fminf(fmaxf(sy * ex, Y0), Y1), dx = fminf(fmaxf(sx * ey, X0), X1);
+  const float qx = fmaf(ex, fmaf(n00, ex, n01x2 * dy), n11 * dy * dy);
+  const float qy = fmaf(ey, fmaf(n11, ey, n01x2 * dx), n00 * dx * dx);
+  return !(fminf(qx, qy) > lim);
+}
 
-// V / (|X - s| amp / sg) of one entry at the lane's two pixels (XX, YY), zero outside the cutoff
-// (k E < c2k); *sgn = amp / sg, the factor the caller accumulates it with.
-template <bool COUNT>
-__device__ __forceinline__ f2 fwd_pair(const float4* en, float xx, f2 YY, float c2k, unsigned& n_cut, float& sgn) {
+// One entry at the lane's two pixels, x and YY = (y, y + 4) from the block centre: their exp2 arguments k E (a
+// pair counts where k E >= c2 k), and V / |X - s| as r 2^(k E).
+struct FwdPair {
+  float ra, rb, ea, eb;
+};
+__device__ __forceinline__ FwdPair fwd_pair(const float4* en, float x, f2 YY) {
   const float4 q0 = en[0], q1 = en[1], q2 = en[2];
-  // the lane's two pixels share their column: the dx terms are scalars
-  const float dx = xx + q1.w;
-  const float aq = q0.x * dx * dx, bq = q0.y * dx, t0 = fmaf(q0.w, dx, q2.y);
-  const f2 DY = f2_add(YY, f2_dup(q2.x));
-  const f2 NUM = f2_fma(DY, f2_fma(f2_dup(q0.z), DY, f2_dup(bq)), f2_dup(aq));  // k num / sg^2
-  const f2 T = f2_fma(f2_dup(q1.x), DY, f2_dup(t0));                             // t / sg
-  const f2 D = f2_fma(T, T, f2_mul(f2_dup(q1.y), NUM));                          // D / sg^2
-  const f2 RS = f2_rsqrt(D);                                                      // sg D^-1/2
-  const f2 ARG = f2_mul(NUM, f2_mul(RS, RS));                                     // k E
-  const f2 VAL = f2_mul(RS, f2_exp2(ARG));
-  float aa, ab, va, vb;
-  f2_unpack(ARG, aa, ab);
-  f2_unpack(VAL, va, vb);
-  const bool ia = aa >= c2k, ib = ab >= c2k;
-  if (COUNT) n_cut += (unsigned)ia + (unsigned)ib;
-  sgn = q1.z;
-  return f2_pack(ia ? va : 0.f, ib ? vb : 0.f);
+  // the lane's two pixels share their column: its terms are formed once
+  const f2 P = f2_fma(f2_dup(x), f2_pack(q0.x, q0.y), f2_pack(q0.z, q0.w));  // x a2 + a1, b0 + x b1
+  float p, bq;
+  f2_unpack(P, p, bq);
+  const float aq = fmaf(x, p, q1.x), tq = fmaf(x, q1.z, q1.y);
+  const f2 NUM = f2_fma(YY, f2_fma(f2_dup(q1.w), YY, f2_dup(bq)), f2_dup(aq));  // k num / sg^2
+  const f2 T = f2_fma(f2_dup(q2.x), YY, f2_dup(tq));                             // t / sg
+  const f2 D = f2_fma(T, T, f2_mul(f2_dup(q2.y), NUM));                          // D / sg^2
+  const f2 RS = f2_rsqrt(D);                                                     // sg D^-1/2
+  const f2 ARG = f2_mul(NUM, f2_mul(RS, RS));                                    // k E
+  FwdPair r;
+  f2_unpack(f2_mul(RS, f2_dup(q2.z)), r.ra, r.rb);
+  f2_unpack(ARG, r.ea, r.eb);
+  return r;
 }
 
-// Each warp walks the tile's whole sorted list in batches of 32: lane l copies record l of the batch
-// into shared memory (cp.async), tests its box against the warp's block and, if they meet, writes the
-// entry to the slot given by the number of meeting lanes below it (so the meeting entries lie packed,
-// in list order); the next batch's copies are then issued and the warp sweeps the packed entries in
-// order (so the sums are deterministic).  No canvas, no atomics, no CTA barrier.
-template <int TS, bool COUNT>
-__global__ void __launch_bounds__(FwdCfg<TS>::threads) k_raster_fwd(
+// Each warp walks the tile's list a batch at a time, one record per lane (in registers, loaded while the batch
+// before it is swept).  A lane tests its record against the warp's blocks and writes the entry of each block
+// that it meets; a ballot's prefix count gives the entry its place, packed and in list order, in the block's
+// table.  The warp then sweeps each block's table in order, four entries per step (independent dependency
+// chains, summed in list order): no canvas, no atomics, no CTA barrier.
+template <int TS, int NB, int SP, bool COUNT>
+__global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP>::min_ctas) k_raster_fwd(
     const float4* __restrict__ grec, const uint32_t* __restrict__ srid, const uint2* __restrict__ ranges,
     const uint32_t* __restrict__ order, const __grid_constant__ ViewsParam views, int tiles_x, int T, int nu, int nv,
-    float c2, float* __restrict__ proj, const float* __restrict__ meas, float* __restrict__ dldi,
-    float* __restrict__ loss_part, float inv_count, unsigned long long* __restrict__ counters) {
-  using C = FwdCfg<TS>;
-  extern __shared__ __align__(16) unsigned char smem[];
+    float* __restrict__ proj, const float* __restrict__ meas, float* __restrict__ dldi,
+    float* __restrict__ loss_part, float c2, float inv_count, unsigned long long* __restrict__ counters) {
+  using C = FwdCfg<TS, NB, SP>;
+  __shared__ float4 tables[C::warps][NB][C::batch * 3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float4* raw = (float4*)smem + (size_t)warp * (C::raw_f4 + C::ent_f4);
-  float4* ent = raw + C::raw_f4;
-  const uint32_t bt = order[blockIdx.x];  // heaviest (projection, tile) lists first
+  const int group = SP == 1 ? warp : warp % C::groups, split = SP == 1 ? 0 : warp / C::groups;
+  const uint32_t bt = order[blockIdx.x / C::subs];  // heaviest (projection, tile) lists first
+  const int sub = blockIdx.x % C::subs;
   const int b = (int)(bt / (uint32_t)T), tile = (int)(bt % (uint32_t)T);
-  const int qx = (tile % tiles_x) * TS + (warp % C::blocks_x) * 8, qy = (tile / tiles_x) * TS + (warp / C::blocks_x) * 8;
-  const int px = qx + (lane & 7), py = qy + (lane >> 3);  // the lane's pixels: (px, py) and (px, py + 4)
-  const float XX = (float)px;
-  const f2 YY = f2_pack((float)py, (float)(py + 4));
+  // first pixel of the warp's first block; block q lies 8 (q mod 2) pixels to the right and 8 (q div 2) below
+  const int gx = (tile % tiles_x) * TS + (sub & 1) * 16 + (NB == 1 ? (group & 1) * 8 : 0);
+  const int gy = (tile / tiles_x) * TS + (sub >> 1) * 16 + (NB == 1 ? group >> 1 : group) * 8;
+  const float cx = (float)gx + 3.5f, cy = (float)gy + 3.5f;  // its centre
+  const float xl = (float)(lane & 7) - 3.5f, yl = (float)(lane >> 3) - 3.5f;
+  const f2 YY = f2_pack(yl, yl + 4.f);
   const uint2 rg = ranges[(size_t)b * T + tile];
   const float c2k = c2 * kNegHalfLog2e;
-  f2 ACC = f2_dup(0.f);
+  float s[NB][2];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) s[q][0] = s[q][1] = 0.f;
   unsigned n_box = 0, n_cut = 0;
-  auto issue = [&](uint32_t k0) {
-    const uint32_t k = k0 + lane;
-    if (k < rg.y) {
-      const float4* src = grec + (size_t)srid[k] * DIGS_REC_F4;
-#pragma unroll
-      for (int q = 0; q < DIGS_REC_F4; ++q) cp_async16(raw + lane * DIGS_REC_F4 + q, src + q);
-    }
-    cp_async_commit();
-  };
-  if (rg.x < rg.y) issue(rg.x);
-  for (uint32_t k0 = rg.x; k0 < rg.y; k0 += C::batch) {
-    cp_async_wait_all();
-    bool meets = false;
+  // lane l's record of the next batch, and the record id one batch further ahead
+  const uint32_t first = rg.x + split * C::batch;
+  uint32_t rid = first + lane < rg.y ? srid[first + lane] : 0u;
+  float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra, rc = ra;
+  auto fetch = [&](uint32_t k0) {
     if (k0 + lane < rg.y) {
-      const float4* r3 = raw + lane * DIGS_REC_F4;
-      const float4 c = r3[2];
-      const int bx = __float_as_int(c.y), by = __float_as_int(c.z);
-      const int x0 = max(bx & 0xffff, qx), x1 = min(bx >> 16, qx + 7);
-      const int y0 = max(by & 0xffff, qy), y1 = min(by >> 16, qy + 7);
-      meets = x0 <= x1 && y0 <= y1;
-      if (COUNT && meets) n_box += (unsigned)((x1 - x0 + 1) * (y1 - y0 + 1));
-      meets = meets && ellipse_meets(r3, x0, x1, y0, y1, c2);
+      const float4* src = grec + (size_t)rid * DIGS_REC_F4;
+      ra = __ldg(src);
+      rb = __ldg(src + 1);
+      rc = __ldg(src + 2);
     }
-    // the meeting entries, compacted in list order: lane -> slot popc(mask below the lane)
-    const unsigned mask = __ballot_sync(0xffffffffu, meets);
-    if (meets) derive_entry(raw + lane * DIGS_REC_F4, ent + __popc(mask & ((1u << lane) - 1u)) * 3);
+    const uint32_t kn = k0 + SP * C::batch + lane;
+    rid = kn < rg.y ? srid[kn] : 0u;
+  };
+  if (first < rg.y) fetch(first);
+  for (uint32_t k0 = first; k0 < rg.y; k0 += SP * C::batch) {
+    const float X = cx - ra.x, Y = cy - ra.y;
+    const float lim = k0 + lane < rg.y ? rc.w : -1.f;  // num >= 0: no record meets nothing
+    const float sy = __fdividef(-0.5f * ra.w, rb.x), sx = __fdividef(-0.5f * ra.w, ra.z);
+    const FwdScaled r = scale_record(ra, rb, rc);
+    int cnt[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      if (COUNT && lim >= 0.f) {
+        const int bx = __float_as_int(rc.y), by = __float_as_int(rc.z);
+        const int qx = gx + (q & 1) * 8, qy = gy + (q >> 1) * 8;
+        const int x0 = max(bx & 0xffff, qx), x1 = min(bx >> 16, qx + 7);
+        const int y0 = max(by & 0xffff, qy), y1 = min(by >> 16, qy + 7);
+        if (x0 <= x1 && y0 <= y1) n_box += (unsigned)((x1 - x0 + 1) * (y1 - y0 + 1));
+      }
+      const float Xq = X + (float)((q & 1) * 8), Yq = Y + (float)((q >> 1) * 8);
+      const bool meets = ellipse_meets(ra.z, ra.w, rb.x, sx, sy, lim, Xq, Yq);
+      const unsigned mask = __ballot_sync(0xffffffffu, meets);
+      if (meets) write_entry(r, Xq, Yq, &tables[warp][q][__popc(mask & ((1u << lane) - 1u)) * 3]);
+      cnt[q] = __popc(mask);
+    }
     __syncwarp();
-    issue(k0 + C::batch);  // lands while this batch is swept
-    const int cnt = __popc(mask);
-    int e = 0;
-    // n entries from e: all evaluated (independent dependency chains), then accumulated in list order
-    auto sweep = [&](int n) {
-      f2 v[8];
-      float sg[8];
+    fetch(k0 + SP * C::batch);  // arrives while this batch is swept
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < n) v[k] = fwd_pair<COUNT>(ent + (e + k) * 3, XX, YY, c2k, n_cut, sg[k]);
+    for (int q = 0; q < NB; ++q) {
+      const float4* e = tables[warp][q];
+      // n entries from e: all evaluated (independent dependency chains), then accumulated in list order
+      auto sweep = [&](int n) {
+        FwdPair v[4];
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < n) ACC = f2_fma(f2_dup(sg[k]), v[k], ACC);
-    };
+        for (int k = 0; k < 4; ++k)
+          if (k < n) v[k] = fwd_pair(e + k * 3, xl, YY);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k < n) {
+            const bool ia = v[k].ea >= c2k, ib = v[k].eb >= c2k;
+            const float va = sfu_exp2(v[k].ea), vb = sfu_exp2(v[k].eb);
+            s[q][0] = ia ? fmaf(v[k].ra, va, s[q][0]) : s[q][0];
+            s[q][1] = ib ? fmaf(v[k].rb, vb, s[q][1]) : s[q][1];
+            if (COUNT) n_cut += (unsigned)ia + (unsigned)ib;
+          }
+        e += n * 3;
+      };
 #pragma unroll 1
-    for (; e + 7 < cnt; e += 8) sweep(8);  // eight entries per step
-    if (e + 3 < cnt) { sweep(4); e += 4; }
-    if (e + 1 < cnt) { sweep(2); e += 2; }
-    if (e < cnt) sweep(1);
+      for (int k = cnt[q] >> 2; k > 0; --k) sweep(4);
+      if (cnt[q] & 2) sweep(2);
+      if (cnt[q] & 1) sweep(1);
+    }
     __syncwarp();
   }
-  cp_async_wait_all();  // the last (empty) group
+  if constexpr (SP > 1) {  // the splits' sums, added in split order by the first
+    float* part = reinterpret_cast<float*>(&tables[0][0][0]);  // [warp][block][2][32]
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      part[((warp * NB + q) * 2) * 32 + lane] = s[q][0];
+      part[((warp * NB + q) * 2 + 1) * 32 + lane] = s[q][1];
+    }
+    __syncthreads();
+    if (split == 0) {
+#pragma unroll
+      for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int z = 1; z < SP; ++z) {
+          s[q][0] += part[(((z * C::groups + group) * NB + q) * 2) * 32 + lane];
+          s[q][1] += part[(((z * C::groups + group) * NB + q) * 2 + 1) * 32 + lane];
+        }
+    }
+  }
   const ViewC& v = views.v[b];
-  float s0, s1;
-  f2_unpack(ACC, s0, s1);
-  float lsum = 0.f;
-  auto emit = [&](int y, float sum) {
-    if (px < nu && y < nv) {
-      const float lp = pixel_ray_length(v, (float)px, (float)y);
-      const float I = sum * lp;
-      const size_t idx = ((size_t)b * nv + y) * nu + px;
-      if (proj) proj[idx] = I;
-      if (meas) {
-        const float res = I - meas[idx];
-        lsum = fmaf(res, res, lsum);
-        if (dldi) dldi[idx] = 2.f * res * inv_count * lp;  // dL/dI * |X - s|, what the backward consumes
+#pragma unroll
+  for (int q = 0; q < NB; ++q) {
+    if (SP > 1 && split != 0) break;
+    const int px = gx + (q & 1) * 8 + (lane & 7);
+    float lsum = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int y = gy + (q >> 1) * 8 + (lane >> 3) + 4 * h;
+      if (px < nu && y < nv) {
+        const float lp = pixel_ray_length(v, (float)px, (float)y);
+        const float I = s[q][h] * lp;
+        const size_t idx = ((size_t)b * nv + y) * nu + px;
+        if (proj) proj[idx] = I;
+        if (meas) {
+          const float res = I - meas[idx];
+          lsum = fmaf(res, res, lsum);
+          if (dldi) dldi[idx] = 2.f * res * inv_count * lp;  // dL/dI * |X - s|, what the backward consumes
+        }
       }
     }
-  };
-  emit(py, s0);
-  emit(py + 4, s1);
+    if (loss_part) {  // one partial per 8 x 8 block
+      lsum = warp_sum(lsum);
+      if (lane == 0) loss_part[(((size_t)b * T + tile) * C::subs + sub) * (C::groups * NB) + group * NB + q] = lsum;
+    }
+  }
   if (COUNT) {
     unsigned c = n_cut, nb = n_box;
 #pragma unroll
@@ -324,10 +375,6 @@ __global__ void __launch_bounds__(FwdCfg<TS>::threads) k_raster_fwd(
       atomicAdd(counters, (unsigned long long)nb);
       atomicAdd(counters + 1, (unsigned long long)c);
     }
-  }
-  if (loss_part) {  // one partial per warp: no CTA barrier
-    lsum = warp_sum(lsum);
-    if (lane == 0) loss_part[((size_t)b * T + tile) * C::warps + warp] = lsum;
   }
 }
 
@@ -587,26 +634,18 @@ __global__ void __launch_bounds__(256) k_gpix(const float* __restrict__ grad_pro
   gpix[idx] = grad_proj[idx] * pixel_ray_length(views.v[b], (float)(p % nu), (float)(p / nu));
 }
 
-template <int TS>
+template <int TS, int NB, int SP>
 static cudaError_t fwd_launch(const Workspace& ws, const ViewsParam& views, float c2, float* proj, const float* meas,
                               float* dldi, float inv_count, bool count, cudaStream_t st) {
-  using C = FwdCfg<TS>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_raster_fwd<TS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
-    cudaFuncSetAttribute(k_raster_fwd<TS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
-    configured = true;
-  }
-  const unsigned grid = (unsigned)ws.T * (unsigned)ws.P;
+  using C = FwdCfg<TS, NB, SP>;
+  const unsigned grid = (unsigned)ws.T * (unsigned)ws.P * C::subs;
   float* lp = meas ? ws.loss_part : nullptr;
   if (count)
-    k_raster_fwd<TS, true><<<grid, C::threads, C::smem, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x,
-                                                              ws.T, ws.nu, ws.nv, c2, proj, meas, dldi, lp, inv_count,
-                                                              ws.counters);
+    k_raster_fwd<TS, NB, SP, true><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
+                                                        ws.nu, ws.nv, proj, meas, dldi, lp, c2, inv_count, ws.counters);
   else
-    k_raster_fwd<TS, false><<<grid, C::threads, C::smem, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views,
-                                                               ws.tiles_x, ws.T, ws.nu, ws.nv, c2, proj, meas, dldi,
-                                                               lp, inv_count, ws.counters);
+    k_raster_fwd<TS, NB, SP, false><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
+                                                         ws.nu, ws.nv, proj, meas, dldi, lp, c2, inv_count, ws.counters);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -615,11 +654,27 @@ cudaError_t launch_raster_fwd(const Workspace& ws, const ViewsParam& views, floa
                               float* dldi, float inv_count, cudaStream_t st) {
   if (ws.P <= 0) return cudaSuccess;
   const bool count = meas == nullptr;  // pair statistics are gathered by plain projections only
+  // How a tile's list is shared out (the sums differ only in rounding).  Splitting it over the CTA's warps cuts
+  // the longest chain of work; it costs a barrier and one more partly filled batch per split.  Four splits are
+  // the faster choice until the launch has a few waves of CTAs by itself (16-pixel tiles, two against four
+  // splits: 16 views of 64^2 0.029 / 0.023 ms, 4096 CTAs of the thorax 0.59 / 0.57, 8192 CTAs of 512^2
+  // 3.85 / 3.77, 10240 CTAs 1.34 / 1.36, 32768 CTAs 4.22 / 4.32; 8-pixel tiles, one against four: 16384 CTAs
+  // 0.59 / 0.56, 40960 CTAs 1.35 / 1.38; 32-pixel tiles, two against four: 10240 CTAs 1.62 / 1.59, 32768 equal).
+  const long long ctas = (long long)ws.P * ws.T * (ws.tile == 32 ? 4 : 1);
+  const bool few = ctas <= (ws.tile == 16 ? 8192 : 16384);
+#define DIGS_FWD(TS, NB, SP) return fwd_launch<TS, NB, SP>(ws, views, c2, proj, meas, dldi, inv_count, count, st)
   switch (ws.tile) {
-    case 8: return fwd_launch<8>(ws, views, c2, proj, meas, dldi, inv_count, count, st);
-    case 16: return fwd_launch<16>(ws, views, c2, proj, meas, dldi, inv_count, count, st);
-    case 32: return fwd_launch<32>(ws, views, c2, proj, meas, dldi, inv_count, count, st);
+    case 8:
+      if (few) DIGS_FWD(8, 1, 4);
+      DIGS_FWD(8, 1, 1);
+    case 16:
+      if (few) DIGS_FWD(16, 2, 4);
+      DIGS_FWD(16, 2, 2);
+    case 32:
+      if (few) DIGS_FWD(32, 2, 4);
+      DIGS_FWD(32, 2, 2);
   }
+#undef DIGS_FWD
   return cudaErrorInvalidValue;
 }
 

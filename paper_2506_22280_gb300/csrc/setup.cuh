@@ -157,14 +157,13 @@ __device__ __forceinline__ bool setup_record(const ViewC& v, const float mu[3], 
   r.wn0 = -s.w0; r.wn1 = -s.w1; r.kappa = s.kappa; r.amp = s.amp;
   r.bx = x0 | (x1 << 16);
   r.by = y0 | (y1 << 16);
-  // Bound on |D - 1| over the box for pairs inside the cutoff: |t - 1| <= tau, kappa num <= kappa c2 D.
-  // When it is small, D^-1/2 = (1 + e)^-1/2 is evaluated by its binomial series through e^3 (truncation
-  // below 35/128 e^4 < 5e-8 for |e| <= 0.02) instead of the SFU's rsqrt.
+  // D over the box for pairs inside the cutoff: |t - 1| <= tau and kappa num <= c2 kappa D, so
+  // D <= (1 + tau)^2 / (1 - c2 kappa), where 1 - c2 kappa = sc > 0 (the source lies outside the cutoff
+  // ellipsoid).
   float mdx = fmaxf(fabsf((float)x0 - s.xc), fabsf((float)x1 - s.xc));
   float mdy = fmaxf(fabsf((float)y0 - s.yc), fabsf((float)y1 - s.yc));
   float tau = fabsf(s.w0) * mdx + fabsf(s.w1) * mdy;
-  float emax = 2.f * tau + tau * tau + 2.f * c2 * s.kappa;
-  r.poly = emax <= 0.02f ? 1 : 0;
+  r.lim = sc > 0.f ? c2 * (1.f + tau) * (1.f + tau) / sc * 1.001f + 1e-4f : __int_as_float(0x7f800000);
   return true;
 }
 
@@ -311,7 +310,7 @@ __device__ __forceinline__ bool ewa_record(const ViewC& v, const float mu[3], co
   r.wn0 = 0.f; r.wn1 = 0.f; r.kappa = 0.f; r.amp = e.amp;
   r.bx = (int)fx0 | ((int)fx1 << 16);
   r.by = (int)fy0 | ((int)fy1 << 16);
-  r.poly = 1;
+  r.lim = c2 * 1.001f + 1e-4f;  // D = 1
   return true;
 }
 
