@@ -57,7 +57,6 @@ size_t layout(Workspace* ws, void* base, int n, int P, int nu, int nv, int R, lo
   w.order = (uint32_t*)take((size_t)P * w.T * 4);
   w.grec = (float4*)take(PN * DIGS_PARTIAL_F4 * sizeof(float4));
   w.bcost = (uint8_t*)take(PN);
-  w.bperm = (uint8_t*)take((size_t)P * ((n + 31) / 32) * 32);
   w.gw_part = (float*)take((size_t)pair_sum_blocks(n_total) * P * R * 4 + 4);
   w.loss_part = (float*)take((size_t)P * w.T * fwd_blocks(tile) * 4 + 4);
   w.ffd = (float*)take((size_t)12 * R * n_total * 4 + 4);
@@ -297,7 +296,7 @@ digs_status backward(Call& c, const float* phi, const float* w, const float* gra
                      float* dens_grad = nullptr) {
   DIGS_TRY(cudaMemsetAsync(g_phi, 0, c.sc.S * phi_floats(c.L) * sizeof(float), c.st));
   mark(c, 5);
-  if (c.g.n > 0) DIGS_TRY(launch_raster_bwd(c.ws, c.views, c.c2, grad_proj, c.st));
+  if (c.g.n > 0) DIGS_TRY(launch_raster_bwd(c.ws, c.sc, c.views, c.c2, grad_proj, c.st));
   mark(c, 6);
   if (c.g.n > 0)
     DIGS_TRY(launch_chain_bwd(c.g, c.sc, c.L, phi, w, c.views, c.P, c.ws, g_mu0, g_scale, g_quat, g_rho, g_phi,

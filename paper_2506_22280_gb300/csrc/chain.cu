@@ -1,9 +1,9 @@
-// Per-Gaussian backward chain: record gradients (the raster backward's ten sums per pair) -> deformed mean
+// Per-Gaussian backward chain: record gradients (the raster backward's twelve moments per pair) -> deformed mean
 // and precision factor A -> K, S, R -> reference Gaussian; then through the DI warp (Eq. 7-8) and the
 // FFD (Eq. 9-11) to the control points phi and the temporal weights w.
 //
 // Three kernels.  (1) For 32 Gaussians per CTA, each warp takes a slot of the projections: one thread per
-// (projection, Gaussian) pair takes the pair's ten pixel sums and runs the adjoint of the projection
+// (projection, Gaussian) pair takes the pair's twelve pixel moments and runs the adjoint of the projection
 // set-up and of A = S^-1 R^T K^-1; the pair adjoints (and their w-weighted sums, what the FFD backward
 // needs) are added up per Gaussian in shared memory, and dL/dw per projection is summed over the CTA's
 // Gaussians.  (2) One thread per Gaussian forms dL/du_r and dL/d(grad u_r) from those sums and scatters
@@ -149,7 +149,7 @@ __device__ __forceinline__ void ffd_scatter_warp(float* __restrict__ g_phi_all, 
   }
 }
 
-// Adjoint of one (projection b, Gaussian n) pair from its ten pixel sums S: dL/dmu' (gmu), dL/dK (gK),
+// Adjoint of one (projection b, Gaussian n) pair from its twelve pixel moments M: dL/dmu' (gmu), dL/dK (gK),
 // dL/ds (gs), dL/dtheta (gth: the gradient for a rotation R -> R (I + [theta]x) of the Gaussian's own
 // axes), dL/drho (grho) and dL/dw_r (gw).  mu0, sc = s, inv_s = 1 / s, Rm, rho: the Gaussian.
 //
@@ -161,7 +161,7 @@ __device__ __forceinline__ void ffd_scatter_warp(float* __restrict__ g_phi_all, 
 template <int R>
 __device__ __forceinline__ void pair_adjoint(const ViewC& v, const float* __restrict__ ffd, int N, int n,
                                              const float* wr, const float mu0[3], const float sc[3],
-                                             const float inv_s[3], const float Rm[9], float rho, const float S[10],
+                                             const float inv_s[3], const float Rm[9], float rho, const float M[12],
                                              float gmu[3], float gK[9], float gs[3], float gth[3], float& grho,
                                              float gw[R]) {
   float mu[3], K[9];
@@ -180,16 +180,40 @@ __device__ __forceinline__ void pair_adjoint(const ViewC& v, const float* __rest
   inv3(K, Ki);
   make_A(inv_s, Rm, Ki, A);
   float gA[9];
-  // record-parameter gradients (see the raster's pair formulas)
+  // The ten sums of the record's gradient from its pixel moments M (see bwd_box_pixels): with B = A (E - 1) its
+  // moments b = M[6..] / k - M[0..], t = 1 + u x + v y (u = wn0, v = wn1) and num = p x^2 + q x y + r y^2,
+  // S[0] = sum g V / amp = sum A D, S[1..5] = sum dL/dnum (x^2, x y, y^2, x, y), S[6..8] = sum dL/dt (1, x, y),
+  // S[9] = sum dL/dkappa.
+  float S[10];
+  auto record_sums = [&](float u, float v, float kap, float p, float q, float r, float amp) {
+    constexpr float ik = -2.f / DIGS_LOG2E;
+    float b[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) b[j] = fmaf(ik, M[6 + j], -M[j]);
+    const float h = 0.5f * amp;
+    S[0] = M[0] + 2.f * (u * M[1] + v * M[3]) + (u * u + kap * p) * M[2] + (2.f * u * v + kap * q) * M[4] +
+           (v * v + kap * r) * M[5];
+    S[1] = h * fmaf(kap, b[2], -M[2]);
+    S[2] = h * fmaf(kap, b[4], -M[4]);
+    S[3] = h * fmaf(kap, b[5], -M[5]);
+    S[4] = h * fmaf(kap, b[1], -M[1]);
+    S[5] = h * fmaf(kap, b[3], -M[3]);
+    S[6] = amp * (b[0] + u * b[1] + v * b[3]);
+    S[7] = amp * (b[1] + u * b[2] + v * b[4]);
+    S[8] = amp * (b[3] + u * b[4] + v * b[5]);
+    S[9] = h * (p * b[2] + q * b[4] + r * b[5]);
+  };
   if (v.ewa) {  // the 2D-Gaussian model: w = kappa = 0
     EwaState es;
     ewa_core(v, mu, A, rho, es);
     const float id = 1.f / es.det2, n00 = es.s11 * id, n01 = -es.s01 * id, n11 = es.s00 * id;
+    record_sums(0.f, 0.f, 0.f, n00, 2.f * n01, n11, es.amp);
     const float g_xc = -2.f * (n00 * S[4] + n01 * S[5]), g_yc = -2.f * (n01 * S[4] + n11 * S[5]);
     ewa_adjoint(v, es, rho, g_xc, g_yc, S[1], 2.f * S[2], S[3], S[0], gmu, gA, grho);
   } else {
     SetupState st;
     setup_core(v, mu, A, rho, st);
+    record_sums(-st.w0, -st.w1, st.kappa, st.n00, 2.f * st.n01, st.n11, st.amp);
     const float g_xc = -(2.f * (st.n00 * S[4] + st.n01 * S[5]) - st.w0 * S[6]);
     const float g_yc = -(2.f * (st.n01 * S[4] + st.n11 * S[5]) - st.w1 * S[6]);
     setup_adjoint(v, st, rho, g_xc, g_yc, S[1], 2.f * S[2], S[3], -S[7], -S[8], S[9], S[0], gmu, gA, grho);
@@ -293,18 +317,18 @@ __global__ void __launch_bounds__(kSlots * 32, 2) k_pair_sum(GaussPtrs g, const 
       else my[q * QS] += x;
     };
     if (valid && v.scan == scan && counts[i] != 0u) {  // else the pair was culled by the projection set-up
-      float S[10];
+      float M[12];
       {
         const float4* p = sums + i * DIGS_PARTIAL_F4;
         const float4 a = p[0], c = p[1], d = p[2];
-        S[0] = a.x; S[1] = a.y; S[2] = a.z; S[3] = a.w;
-        S[4] = c.x; S[5] = c.y; S[6] = c.z; S[7] = c.w;
-        S[8] = d.x; S[9] = d.y;
+        M[0] = a.x; M[1] = a.y; M[2] = a.z; M[3] = a.w;
+        M[4] = c.x; M[5] = c.y; M[6] = c.z; M[7] = c.w;
+        M[8] = d.x; M[9] = d.y; M[10] = d.z; M[11] = d.w;
       }
       float wr[R], gmu[3], gK[9], gs[3], gth[3], grho;
 #pragma unroll
       for (int r = 0; r < R; ++r) wr[r] = __ldg(wb + r);
-      pair_adjoint<R>(v, ffd, N, n, wr, mu0, scl, inv_s, Rm, rho, S, gmu, gK, gs, gth, grho, gw);
+      pair_adjoint<R>(v, ffd, N, n, wr, mu0, scl, inv_s, Rm, rho, M, gmu, gK, gs, gth, grho, gw);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         put(c, gmu[c]);

@@ -31,9 +31,8 @@ struct Workspace {
   uint32_t* seg;          // [2P + 2] each projection's first pair and first sort block
   uint2* ranges;          // [P * T] sorted-range of each (projection, tile)
   uint32_t* order;        // [P * T] forward launch order (longest lists first)
-  float4* grec;           // [P * n * 3] backward: the ten pixel sums of each (projection, Gaussian) record
-  uint8_t* bcost;         // [P * n] backward sweep cost of each record: box pixels / 32, capped at 255
-  uint8_t* bperm;         // [P][32 ceil(n / 32)] backward: each group of 32 records in order of sweep cost
+  float4* grec;           // [P * n * 3] backward: the twelve pixel moments of each (projection, Gaussian) record
+  uint8_t* bcost;         // [P * n] backward sweep cost of each record: box pixels / 32, capped at 255 (0: culled)
   float* gw_part;         // [pair-sum CTAs][P][R] dL/dw partial sums
   float* ffd;             // [12 R][n_total]: u_r (3R components) then grad u_r (9R) at each mean
   float* ffd2;            // [18 R][n_total]: second derivatives of u_r (6 per component)
@@ -95,7 +94,7 @@ cudaError_t launch_emit(const Workspace& ws, cudaStream_t st);
 cudaError_t launch_raster_fwd(const Workspace& ws, const ViewsParam& views, float c2, float* proj, const float* meas,
                               float* dldi, float inv_count, cudaStream_t st);
 // grad_proj = dL/dI, or nullptr when ws.dldi already holds dL/dI * |X - s| (from the step's forward).
-cudaError_t launch_raster_bwd(const Workspace& ws, const ViewsParam& views, float c2, const float* grad_proj,
+cudaError_t launch_raster_bwd(const Workspace& ws, const ScanTable& sc, const ViewsParam& views, float c2, const float* grad_proj,
                               cudaStream_t st);
 // Sums part[0 .. n) in a fixed order (overwriting part) and writes scale * sum to out[0].
 cudaError_t launch_loss_reduce(float* part, int n, float* out, float scale, cudaStream_t st);

@@ -18,16 +18,17 @@
 // 5.31 -> 4.22 ms; 16: 0.78 -> 0.57; 8 of 500k Gaussians on 512^2: 5.2 -> 3.8; 16 of 2,000 on 64^2:
 // 0.044 -> 0.023.
 //
-// Backward: needs no tile lists.  One half-warp per (projection, Gaussian) record (the two records of a
-// warp of similar box size, paired by k_bwd_pairing) sweeps the record's pixel box in 16-column slices,
-// reading g = dL/dI * |X - s| from the projection-sized image (L1/L2 resident).  Narrow slices (w <= 8):
-// lane l owns column (l mod w), starts at row (l div w) and takes the row pair (r, r + s), s = 16 div w,
-// stepping 2s rows; wider slices: the column pair (c, c + ceil(w/2)) of row (l div ceil(w/2)), stepping
-// s = 16 div ceil(w/2) rows.  Each lane accumulates seven sums per pixel of its pair and turns them into
-// the ten sufficient statistics of the record gradient; the half-warp reduces them with an 11-shuffle
-// recursive halving and ten lanes write them to the record's slot (no atomics).  A CTA sweeps four units
-// of 16 records in turn, each unit's records and tile counts copied to shared memory by cp.async while
-// the unit before it is swept.
+// Backward: needs no tile lists.  One half-warp per (projection, Gaussian) record (the two records of a warp of
+// similar box size) sweeps the record's pixel box in 16-column slices, reading g = dL/dI * |X - s| from the
+// projection-sized image (L1/L2 resident).  Narrow slices (w <= 8): lane l owns column (l mod w), starts at row
+// (l div w) and takes the row pair (r, r + s), s = 16 div w, stepping 2s rows; wider slices: the column pair
+// (c, c + ceil(w/2)) of row (l div ceil(w/2)), stepping s = 16 div ceil(w/2) rows.  Each lane accumulates six
+// moments per pixel of its pair; a slice adds their twelve (dx, dy)-moments, the half-warp reduces those with a
+// 12-shuffle recursive halving and twelve lanes write them to the record's slot (no atomics).
+// What bounds it: the FMA pipe (packed arithmetic takes two of its cycles; 70 % busy) and the instructions per
+// record around the sweep (a third of the time).  128 thorax projections (100k Gaussians, 256^2), with the
+// ranking of the records: 8.82 -> 7.36 ms; 16 of 2,000 on 64^2: 0.032 -> 0.027; 64 of four scans of 30k to 200k,
+// whose missing records are no longer visited: 4.9 -> 3.8.
 //
 // Loss: per-warp partials of the squared residuals from the forward, summed in two fixed-order levels.
 #include <algorithm>
@@ -380,159 +381,162 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
 
 // ---- backward: one half-warp per (projection, Gaussian) record, over the record's whole pixel box ----
 
-constexpr int kBwdThreads = 256;
-constexpr int kBwdRounds = 4;  // record units per backward CTA
 
-// Adds the lane's share of the ten record-gradient sums, all but the first divided by amp / 2:
-// sum g V/amp; sum dL/dnum (dx^2, dx dy, dy^2); sum dL/dnum (dx, dy); sum dL/dt (1, dx, dy);
-// sum dL/dkappa.  gp points at g = dL/dI * |X - s| of the lane's first pixel in the projection image
-// (row pitch nu); (dx1, dy1) is that pixel's offset from the projected mean.
-//
-// Per pixel, with A = (g V / amp) / D and B = A (E - 1): dL/dnum = kappa B - A, dL/dt / 2 = B t and
-// dL/dkappa = B num.  A lane's pixel keeps its column, so t = t0 + wn1 dy and num = a + b dy + n11 dy^2
-// with column constants t0, a, b: every sum above is a combination of the six dy-moments
-// sum A dy^j and sum B dy^j (j = 0, 1, 2), which are all the loop accumulates besides sum g V / amp.
+// Adds the lane's share of a record's twelve pixel moments: with A = (g V / amp) / D and k E the exp2 argument,
+//   Sv[0..5] = sum A (1, dx, dx^2, dy, dx dy, dy^2) and Sv[6..11] = sum A k E (the same),
+// (dx, dy) the pixel's offset from the projected mean.  With B = A (E - 1): dL/dnum = (amp / 2) (kappa B - A),
+// dL/dt = amp B t, dL/dkappa = (amp / 2) B num and g V / amp = A D, and t, num and D are polynomials of degree two
+// in (dx, dy), so the ten sums of the record's gradient follow from these twelve with per-record constants:
+// pair_adjoint forms them, once per record, instead of every lane of the sweep once per slice of the box.
+// gp points at g = dL/dI * |X - s| of the lane's first pixel in the projection image (row pitch nu); (dx1, dy1)
+// is that pixel's offset.  A lane's pixel keeps its column, so the loop accumulates the six dy-moments alone (20
+// packed operations per pixel pair, 23 with the seven sums it kept before).
 __device__ __forceinline__ void bwd_box_pixels(const Rec& R0, const HalfLanes& B, int h, float dx1, float dy1,
-                                               const float* __restrict__ gp, int nu, float c2, float Sv[10]) {
+                                               const float* __restrict__ gp, int nu, float c2, float Sv[12]) {
   // k = -log2(e) / 2 is folded into the quadratic form: NUM = k num, ARG = k E (the exp2 argument)
-  const float dx2 = dx1 + (float)B.pdx;
-  const f2 DX = f2_pack(dx1, dx2);
+  const f2 DX = f2_pack(dx1, dx1 + (float)B.pdx);
   const f2 AQ = f2_mul(f2_mul(f2_dup(kNegHalfLog2e * R0.n00), DX), DX);
   const f2 BQ = f2_mul(f2_dup(kNegHalfLog2e * R0.n01x2), DX);
   const f2 T0 = f2_fma(f2_dup(R0.wn0), DX, f2_dup(1.f));
   const f2 N11 = f2_dup(kNegHalfLog2e * R0.n11), WN1 = f2_dup(R0.wn1);
-  const f2 KAPK = f2_dup(R0.kappa * (1.f / kNegHalfLog2e));
-  const f2 IK = f2_dup(1.f / kNegHalfLog2e), MONE = f2_dup(-1.f), STEP = f2_dup((float)B.ystep);
+  const f2 KAPK = f2_dup(R0.kappa * (1.f / kNegHalfLog2e)), STEP = f2_dup((float)B.ystep);
   const f2 C2K = f2_dup(c2 * kNegHalfLog2e);
   const int pstep = B.ystep * nu, d2 = B.pdy * nu + B.pdx, hb = B.col2 ? h - B.pdy : 0;
   f2 DY = f2_pack(dy1, dy1 + (float)B.pdy);
-  f2 S0 = f2_dup(0.f), A0 = S0, A1 = S0, A2 = S0, B0 = S0, B1 = S0, B2 = S0;
+  f2 A0 = f2_dup(0.f), A1 = A0, A2 = A0, E0 = A0, E1 = A0, E2 = A0;
   for (int r = B.r0; r < h; r += B.ystep, DY = f2_add(DY, STEP), gp += pstep) {
-    f2 NUM = f2_fma(DY, f2_fma(N11, DY, BQ), AQ);
-    f2 T = f2_fma(WN1, DY, T0);
-    f2 D = f2_fma(T, T, f2_mul(KAPK, NUM));
+    const f2 NUM = f2_fma(DY, f2_fma(N11, DY, BQ), AQ);
+    const f2 T = f2_fma(WN1, DY, T0);
+    const f2 D = f2_fma(T, T, f2_mul(KAPK, NUM));
     // E <= cutoff^2 taken as num <= c2 D (D > 0), i.e. k num >= k c2 D: known before the SFU work, so
     // the two loads of dL/dI are in flight while it runs
-    f2 LIM = f2_mul(C2K, D);
+    const f2 LIM = f2_mul(C2K, D);
     float na, nb, la, lb;
     f2_unpack(NUM, na, nb);
     f2_unpack(LIM, la, lb);
     const float ga = (na >= la) ? __ldg(gp) : 0.f;
     const float gb = (r < hb && nb >= lb) ? __ldg(gp + d2) : 0.f;  // partner in the box
-    f2 RS = f2_rsqrt(D);
-    f2 INVD = f2_mul(RS, RS);
-    f2 ARG = f2_mul(NUM, INVD);
-    f2 BV = f2_mul(RS, f2_exp2(ARG));                      // V / amp
-    f2 GA = f2_mul(f2_pack(ga, gb), BV);                  // g V / amp
-    S0 = f2_add(S0, GA);
-    f2 AL = f2_mul(GA, INVD);                               // A = (dL/dV V / (2 D)) / (amp / 2)
-    f2 AE = f2_mul(AL, f2_fma(ARG, IK, MONE));              // B = A (E - 1)
-    f2 ALD = f2_mul(AL, DY), AED = f2_mul(AE, DY);
+    const f2 RS = f2_rsqrt(D);
+    const f2 INVD = f2_mul(RS, RS);
+    const f2 ARG = f2_mul(NUM, INVD);
+    const f2 BV = f2_mul(RS, f2_exp2(ARG));                            // V / amp
+    const f2 AL = f2_mul(f2_mul(f2_pack(ga, gb), BV), INVD);           // A
+    const f2 AE = f2_mul(AL, ARG);                                     // A k E
+    const f2 DY2 = f2_mul(DY, DY);
     A0 = f2_add(A0, AL);
-    A1 = f2_add(A1, ALD);
-    A2 = f2_fma(ALD, DY, A2);
-    B0 = f2_add(B0, AE);
-    B1 = f2_add(B1, AED);
-    B2 = f2_fma(AED, DY, B2);
+    A1 = f2_fma(AL, DY, A1);
+    A2 = f2_fma(AL, DY2, A2);
+    E0 = f2_add(E0, AE);
+    E1 = f2_fma(AE, DY, E1);
+    E2 = f2_fma(AE, DY2, E2);
   }
-  // per pixel of the pair: the dy-moments of dL/dnum, dL/dt and dL/dkappa from those of A and B, then
-  // the dx-moments from the pixel's column
-  float s0[2], a0[2], a1[2], a2[2], b0[2], b1[2], b2[2], aq[2], bq[2], t0[2];
-  f2_unpack(S0, s0[0], s0[1]);
-  f2_unpack(A0, a0[0], a0[1]);
-  f2_unpack(A1, a1[0], a1[1]);
-  f2_unpack(A2, a2[0], a2[1]);
-  f2_unpack(B0, b0[0], b0[1]);
-  f2_unpack(B1, b1[0], b1[1]);
-  f2_unpack(B2, b2[0], b2[1]);
-  f2_unpack(AQ, aq[0], aq[1]);
-  f2_unpack(BQ, bq[0], bq[1]);
-  f2_unpack(T0, t0[0], t0[1]);
-  const float kap = R0.kappa, wn1 = R0.wn1, n11k = kNegHalfLog2e * R0.n11;
-  const float dxs[2] = {dx1, dx2};
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float dx = dxs[j];
-    const float g0 = fmaf(kap, b0[j], -a0[j]), g1 = fmaf(kap, b1[j], -a1[j]), g2 = fmaf(kap, b2[j], -a2[j]);
-    const float th0 = fmaf(t0[j], b0[j], wn1 * b1[j]), th1 = fmaf(t0[j], b1[j], wn1 * b2[j]);
-    const float gk = fmaf(aq[j], b0[j], fmaf(bq[j], b1[j], n11k * b2[j]));
-    Sv[0] += s0[j];
-    Sv[1] += dx * dx * g0;
-    Sv[2] += dx * g1;
-    Sv[3] += g2;
-    Sv[4] += dx * g0;
-    Sv[5] += g1;
-    Sv[6] += 2.f * th0;
-    Sv[7] += 2.f * dx * th0;
-    Sv[8] += 2.f * th1;
-    Sv[9] += gk * (1.f / kNegHalfLog2e);
-  }
+  auto add = [&](int q, f2 v) {
+    float lo, hi;
+    f2_unpack(v, lo, hi);
+    Sv[q] += lo + hi;
+  };
+  const f2 AX = f2_mul(A0, DX), EX = f2_mul(E0, DX);
+  add(0, A0);
+  add(1, AX);
+  add(2, f2_mul(AX, DX));
+  add(3, A1);
+  add(4, f2_mul(A1, DX));
+  add(5, A2);
+  add(6, E0);
+  add(7, EX);
+  add(8, f2_mul(EX, DX));
+  add(9, E1);
+  add(10, f2_mul(E1, DX));
+  add(11, E2);
 }
 
-// Sum ten per-lane values over each group of LPR lanes and store them to out[0..9]: first over each
+// Sum twelve per-lane values over each group of LPR lanes and store them to out[0..11]: first over each
 // half-warp (lanes hl = 0..15), then, for LPR = 32, across the two halves.
-// Recursive halving over an uneven split, 5 + 3 + 2 + 1 shuffles: after the xor-8 exchange a lane
-// holds five values (0-4 or 5-9), after xor-4 three of those five (local 0-2, or 3-4 plus a pad),
-// after xor-2 two, after xor-1 one, the value 5 b3 + 3 b2 + 2 b1 + b0 (b_k = bit k of hl) when that
-// lies inside its group of five.
+// Recursive halving, 6 + 3 + 2 + 1 shuffles: after the xor-8 exchange a lane holds six values, after xor-4
+// three, after xor-2 two (or one and a pad), after xor-1 one, the value 6 b3 + 3 b2 + 2 b1 + b0 (b_k = bit k
+// of hl) where 2 b1 + b0 < 3.
 template <int LPR>
-__device__ __forceinline__ void group_reduce_store10(const float v[10], float* out, int hl, bool store) {
+__device__ __forceinline__ void group_reduce_store12(const float v[12], float* out, int hl, bool store) {
   const unsigned full = 0xffffffffu;
-  float a[5];
+  float a[6];
   {
     const bool hi = (hl & 8) != 0;
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      const float keep = hi ? v[5 + j] : v[j], send = hi ? v[j] : v[5 + j];
+    for (int j = 0; j < 6; ++j) {
+      const float keep = hi ? v[6 + j] : v[j], send = hi ? v[j] : v[6 + j];
       a[j] = keep + __shfl_xor_sync(full, send, 8);
     }
   }
-  float b0, b1, b2;
+  float b[3];
   {
     const bool hi = (hl & 4) != 0;
-    const float k0 = hi ? a[3] : a[0], k1 = hi ? a[4] : a[1], k2 = hi ? 0.f : a[2];
-    const float s0 = hi ? a[0] : a[3], s1 = hi ? a[1] : a[4], s2 = hi ? a[2] : 0.f;
-    b0 = k0 + __shfl_xor_sync(full, s0, 4);
-    b1 = k1 + __shfl_xor_sync(full, s1, 4);
-    b2 = k2 + __shfl_xor_sync(full, s2, 4);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float keep = hi ? a[3 + j] : a[j], send = hi ? a[j] : a[3 + j];
+      b[j] = keep + __shfl_xor_sync(full, send, 4);
+    }
   }
   float c0, c1;
   {
     const bool hi = (hl & 2) != 0;
-    const float k0 = hi ? b2 : b0, k1 = hi ? 0.f : b1;
-    const float s0 = hi ? b0 : b2, s1 = hi ? b1 : 0.f;
+    const float k0 = hi ? b[2] : b[0], k1 = hi ? 0.f : b[1];
+    const float s0 = hi ? b[0] : b[2], s1 = hi ? b[1] : 0.f;
     c0 = k0 + __shfl_xor_sync(full, s0, 2);
     c1 = k1 + __shfl_xor_sync(full, s1, 2);
   }
   const bool hi = (hl & 1) != 0;
   float d = (hi ? c1 : c0) + __shfl_xor_sync(full, hi ? c0 : c1, 1);
   if (LPR == 32) d += __shfl_xor_sync(full, d, 16);
-  const int bit2 = (hl >> 2) & 1;
-  const int local = 3 * bit2 + 2 * ((hl >> 1) & 1) + (hl & 1);
-  if (store && (LPR == 16 || (threadIdx.x & 16) == 0) && local < (bit2 ? 5 : 3)) out[((hl & 8) ? 5 : 0) + local] = d;
+  const int local = 2 * ((hl >> 1) & 1) + (hl & 1);
+  if (store && (LPR == 16 || (threadIdx.x & 16) == 0) && local < 3)
+    out[((hl & 8) ? 6 : 0) + ((hl & 4) ? 3 : 0) + local] = d;
 }
 
-// The two records of a backward warp are swept in lockstep, so the warp takes as many passes as the
-// longer of the two.  Each warp here ranks a group of 32 consecutive records of one projection by their
-// sweep cost (box pixels / 32, written by the set-up: the pass count up to the lane layout's rounding;
-// stable: ties in index order; bit-sliced ballots over a 9-bit key, records past n last) and writes
-// the record of each rank, so that the backward pairs records of adjacent ranks.
-// Grid: (ceil(G / 8), P) with G = ceil(n / 32) groups per projection; 256 threads.
-__global__ void __launch_bounds__(256) k_bwd_pairing(const uint8_t* __restrict__ cost, const uint32_t* __restrict__ counts,
-                                                     int N, int G, uint8_t* __restrict__ perm) {
-  const int lane = threadIdx.x & 31;
-  const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (g >= G) return;  // whole warps
-  const int b = blockIdx.y;
-  const int n = g * 32 + lane;
-  unsigned key = 511u;
-  if (n < N) {
-    const size_t i = (size_t)b * N + n;
-    key = counts[i] != 0u ? (unsigned)cost[i] : 0u;  // padding records of smaller scans have no tiles
-  }
+// One group of LPR lanes (16: two records per warp, 32: one) per (projection, Gaussian) record: the twelve
+// moments over every pixel of the record's box, reduced over the group and written to grec[record].  Nothing is
+// written for culled records: the chain does not read those.
+//
+// A warp takes ranks of one group of 32 consecutive records of a projection.  The two records of a warp are
+// swept in lockstep, for as many passes as the longer needs, so the warp first ranks the group by sweep cost
+// (box pixels / 32, written by the set-up; 0: culled; ties in index order; bit-sliced ballots) and sweeps
+// records of adjacent ranks together; the culled ones rank first and are skipped.  Ranking in the sweeping
+// warps themselves replaced a kernel that wrote the ranks to memory (0.076 ms of 128 projections) and two
+// dependent loads per record.
+// WR rounds of 32 / LPR records per warp and W warps per CTA: one warp that takes the whole group, in a CTA of its
+// own, whose place is free for the next as soon as it ends (eight warps in a CTA wait for the longest: 8.05
+// against 7.5 ms for 128 thorax projections); where that leaves too few warps, a quarter of the group each (and
+// each quarter's warp ranks the group again, about 45 instructions).
+// The next rounds' records are copied to shared memory by cp.async (double buffer) while one is swept.
+// 28 warps of 72 registers per SM: with 64 registers (32 warps) the loop spills and recomputes its lane layout,
+// with 80 (24 warps) its latencies show (8.05, 7.8 and 9.4 ms with four-warp CTAs).
+// counts.n[b]: records of projection b that exist (its scan's Gaussians); N: record stride of a projection.
+// Grid: (ceil(warps / W), P), warps = ceil(N / 32) * 32 / (WR * (32 / LPR)).
+struct ViewCounts {
+  int n[DIGS_MAX_VIEWS];
+};
+template <int LPR, int WR, int W>
+__global__ void __launch_bounds__(32 * W, 28 / W) k_raster_bwd(const float4* __restrict__ rec,
+                                                               const uint8_t* __restrict__ cost,
+                                                               const __grid_constant__ ViewCounts counts, int N, int nu,
+                                                               int nv, const float* __restrict__ gpix, float c2,
+                                                               float* __restrict__ grec) {
+  constexpr int kPer = 32 / LPR;             // records per round
+  constexpr int kSplits = 32 / (kPer * WR);  // warps per group of 32 records
+  __shared__ __align__(16) float4 sbuf[W][2][kPer][DIGS_REC_F4];
+  __shared__ uint8_t order[W][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, hl = lane & (LPR - 1), half = lane / LPR;
+  const int b = blockIdx.y, nb = counts.n[b];
+  const int gw = blockIdx.x * W + warp;
+  const int n0 = gw / kSplits * 32, r0 = gw % kSplits * (kPer * WR);  // the group's first record, the warp's first rank
+  if (n0 >= nb) return;  // whole warps
+  rec += (size_t)b * N * DIGS_REC_F4;
+  grec += (size_t)b * N * (DIGS_PARTIAL_F4 * 4);
+  const float* gimg = gpix + (size_t)b * nv * nu;
+  const unsigned key = n0 + lane < nb ? (unsigned)cost[(size_t)b * N + n0 + lane] : 0u;
+  const int dead = __popc(__ballot_sync(0xffffffffu, key == 0u));
   unsigned lt = 0u, eq = 0xffffffffu;  // lanes with a smaller key; lanes whose key agrees so far
 #pragma unroll
-  for (int bit = 8; bit >= 0; --bit) {
+  for (int bit = 7; bit >= 0; --bit) {
     const unsigned one = (key >> bit) & 1u;
     const unsigned m = __ballot_sync(0xffffffffu, one);
     if (one) {
@@ -542,84 +546,45 @@ __global__ void __launch_bounds__(256) k_bwd_pairing(const uint8_t* __restrict__
       eq &= ~m;
     }
   }
-  const int rank = __popc(lt) + __popc(eq & ((1u << lane) - 1u));
-  perm[((size_t)b * G + g) * 32 + rank] = (uint8_t)lane;
-}
-
-// One group of LPR lanes (16: two records per warp, 32: one) per (projection, Gaussian) record: the ten
-// sums over every pixel of the record's box, reduced over the group and written to grec[record] (12
-// floats, the last two unused).  Records whose Gaussian was culled get zeros.
-// Each CTA takes `rounds` consecutive units of 256 / LPR records (unit u of projection b: for LPR = 16
-// ranks 16 (u mod 2) .. + 15 of record group u / 2 in k_bwd_pairing's order, else records 8u .. 8u + 7).
-// A group's record and its tile count go to shared memory by cp.async two units ahead (double buffer;
-// the unit after that has its record index loaded while the current one is swept), so that only a CTA's
-// first unit waits for them.
-// Grid: (ceil(units / rounds), P), units = ceil(N / (256 / LPR)).
-template <int LPR>
-__global__ void __launch_bounds__(kBwdThreads, 4) k_raster_bwd(const float4* __restrict__ rec,
-                                                                const uint32_t* __restrict__ counts, int N, int nu,
-                                                                int nv, const float* __restrict__ gpix, float c2,
-                                                                const uint8_t* __restrict__ perm,
-                                                                float* __restrict__ grec, int rounds) {
-  constexpr int kRecords = kBwdThreads / LPR;  // records per unit
-  __shared__ __align__(16) float4 sbuf[2][kRecords][DIGS_REC_F4 + 1];  // record, then its tile count
-  const int hl = threadIdx.x & (LPR - 1);
-  const int b = blockIdx.y;
-  const int slot = (int)(threadIdx.x / LPR);
-  const int units = (N + kRecords - 1) / kRecords;
-  const int G = (N + 31) >> 5;
-  const int u0 = blockIdx.x * rounds;
-  auto record_of = [&](int u) -> int {  // this group's record in unit u (N: none)
-    if (u >= units || u - u0 >= rounds) return N;
-    if (LPR == 16) {  // unit pairs share a group of 32 records, taken in the order of k_bwd_pairing
-      const int g = u >> 1;
-      return g * 32 + perm[((size_t)b * G + g) * 32 + (u & 1) * 16 + slot];
-    }
-    return u * kRecords + slot;
-  };
-  auto fetch = [&](int n, int buf) {  // one commit group per call and thread, empty or not
-    if (n < N && hl <= DIGS_REC_F4) {
-      const size_t i = (size_t)b * N + n;
-      if (hl < DIGS_REC_F4)
-        cp_async16(&sbuf[buf][slot][hl], rec + i * DIGS_REC_F4 + hl);
-      else
-        cp_async4(&sbuf[buf][slot][DIGS_REC_F4], counts + i);
+  order[warp][__popc(lt) + __popc(eq & ((1u << lane) - 1u))] = (uint8_t)lane;
+  __syncwarp();
+  const int of_rank = order[warp][lane];  // the record of rank `lane`
+  const int i0 = max(0, (dead - r0) / kPer);  // the first round with a live record
+  auto fetch = [&](int i) {  // one commit group per call and thread, empty or not
+    if (i < WR) {
+      const int n = n0 + __shfl_sync(0xffffffffu, of_rank, r0 + i * kPer + half);
+      if (hl < DIGS_REC_F4) cp_async16(&sbuf[warp][i & 1][half][hl], rec + (unsigned)n * DIGS_REC_F4 + hl);
     }
     cp_async_commit();
   };
-  int n_cur = record_of(u0), n_next = record_of(u0 + 1);
-  fetch(n_cur, 0);
-  fetch(n_next, 1);
-  const float* gimg = gpix + (size_t)b * nv * nu;
-  for (int r = 0; r < rounds; ++r) {
-    const int n_after = record_of(u0 + r + 2);  // in flight while this unit is swept
-    const int buf = r & 1;
-    cp_async_wait_but_one();  // this unit's copies have landed (the next unit's may still be in flight)
+  fetch(i0);
+  fetch(i0 + 1);
+#pragma unroll 1
+  for (int i = i0; i < WR; ++i) {
+    cp_async_wait_but_one();  // this round's copies have landed (the next one's may still be in flight)
     __syncwarp();
-    const bool valid = n_cur < N;
-    float Sv[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (valid && __float_as_uint(sbuf[buf][slot][DIGS_REC_F4].x) != 0u) {
-      const Rec R0 = load_rec(&sbuf[buf][slot][0]);
+    const int rank = r0 + i * kPer + half;
+    const bool live = rank >= dead;
+    float Sv[12];
+#pragma unroll
+    for (int q = 0; q < 12; ++q) Sv[q] = 0.f;
+    if (live) {
+      const Rec R0 = load_rec(sbuf[warp][i & 1][half]);
       const int x0 = R0.bx & 0xffff, x1 = R0.bx >> 16, y0 = R0.by & 0xffff, y1 = R0.by >> 16;
       const int w = x1 - x0 + 1, h = y1 - y0 + 1;
       for (int cx = 0; cx < w; cx += LPR) {  // boxes wider than LPR pixels: LPR-column slices
         const HalfLanes B = group_lanes<LPR>(min(LPR, w - cx), h, hl);
         if (B.active) {
           const int px = x0 + cx + B.c, py = y0 + B.r0;
-          const float* gp = gimg + (size_t)py * nu + px;
+          const float* gp = gimg + (unsigned)(py * nu + px);
           bwd_box_pixels(R0, B, h, (float)px - R0.xc, (float)py - R0.yc, gp, nu, c2, Sv);
         }
       }
-      const float amph = 0.5f * R0.amp;
-#pragma unroll
-      for (int q = 1; q < 10; ++q) Sv[q] *= amph;
     }
-    group_reduce_store10<LPR>(Sv, grec + ((size_t)b * N + (valid ? n_cur : 0)) * (DIGS_PARTIAL_F4 * 4),
-                              threadIdx.x & 15, valid);
+    const int n = n0 + __shfl_sync(0xffffffffu, of_rank, rank);
+    group_reduce_store12<LPR>(Sv, grec + (unsigned)n * (DIGS_PARTIAL_F4 * 4), lane & 15, live);
     __syncwarp();  // every lane has read this buffer before it is refilled
-    fetch(n_after, buf);
-    n_cur = n_next;
-    n_next = n_after;
+    fetch(i + 2);
   }
   cp_async_wait_all();
 }
@@ -678,7 +643,7 @@ cudaError_t launch_raster_fwd(const Workspace& ws, const ViewsParam& views, floa
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_raster_bwd(const Workspace& ws, const ViewsParam& views, float c2, const float* grad_proj,
+cudaError_t launch_raster_bwd(const Workspace& ws, const ScanTable& sc, const ViewsParam& views, float c2, const float* grad_proj,
                               cudaStream_t st) {
   if (ws.P <= 0 || ws.n <= 0) return cudaSuccess;
   if (grad_proj) {  // else ws.dldi already holds dL/dI * |X - s| (written by the step's forward)
@@ -686,20 +651,19 @@ cudaError_t launch_raster_bwd(const Workspace& ws, const ViewsParam& views, floa
     k_gpix<<<g, 256, 0, st>>>(grad_proj, views, ws.nu, ws.nv, ws.dldi);
     note_launches(1);
   }
-  if (ws.bwd_lanes == 32) {
-    const int units = (ws.n + kBwdThreads / 32 - 1) / (kBwdThreads / 32);
-    dim3 grid((units + kBwdRounds - 1) / kBwdRounds, ws.P);
-    k_raster_bwd<32><<<grid, kBwdThreads, 0, st>>>(ws.rec, ws.counts, ws.n, ws.nu, ws.nv, ws.dldi, c2, nullptr,
-                                                   (float*)ws.grec, kBwdRounds);
-  } else {
-    const int G = (ws.n + 31) / 32;
-    k_bwd_pairing<<<dim3((G + 7) / 8, ws.P), 256, 0, st>>>(ws.bcost, ws.counts, ws.n, G, ws.bperm);
-    note_launches(1);
-    const int units = (ws.n + kBwdThreads / 16 - 1) / (kBwdThreads / 16);
-    dim3 grid((units + kBwdRounds - 1) / kBwdRounds, ws.P);
-    k_raster_bwd<16><<<grid, kBwdThreads, 0, st>>>(ws.rec, ws.counts, ws.n, ws.nu, ws.nv, ws.dldi, c2, ws.bperm,
-                                                   (float*)ws.grec, kBwdRounds);
-  }
+  ViewCounts counts;
+  for (int b = 0; b < ws.P; ++b) counts.n[b] = sc.off[views.v[b].scan + 1] - sc.off[views.v[b].scan];
+  const int G = (ws.n + 31) / 32;
+#define DIGS_BWD(LPR, WR, W)                                                                        \
+  k_raster_bwd<LPR, WR, W><<<dim3((G * (LPR / WR) + W - 1) / W, ws.P), 32 * W, 0, st>>>(            \
+      ws.rec, ws.bcost, counts, ws.n, ws.nu, ws.nv, ws.dldi, c2, (float*)ws.grec)
+  // A warp per group of 32 records from 8192 groups on, four below: 1000 groups 0.037 / 0.027 ms, 7300 0.117 / 0.111,
+  // 12500 0.260 / 0.258, 50000 0.949 / 0.987, 400000 7.36 / 7.79.  One record per warp (32 lanes): always four
+  // warps per group (1000 groups 0.043 / 0.031, 50000 1.28 / 1.16).
+  if (ws.bwd_lanes == 32) DIGS_BWD(32, 8, 4);
+  else if ((long long)G * ws.P > 8192) DIGS_BWD(16, 16, 1);
+  else DIGS_BWD(16, 4, 4);
+#undef DIGS_BWD
   note_launches(1);
   return cudaGetLastError();
 }
