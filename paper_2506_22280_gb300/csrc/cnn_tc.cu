@@ -3,24 +3,14 @@
 //
 // Activations live in BF16, NHWC, exactly as the GEMMs consume them: the post-ReLU output of every
 // convolution is rounded once by the epilogue that produces it (the rounding the tensor cores would
-// apply anyway), its sign is the ReLU mask of the backward.  Every GEMM is one launch of one kernel
-// template: 128 threads per CTA, looping over 128-row tiles of C; the four warps fill a ring of 2-4 stages of 64-deep K slices of
-// A and B with 16-byte cp.async copies (zero-filled where an operand is padding), one thread issues the
-// four 128 x BN x 16 MMAs of a slice and commits them to the slice's mbarrier, and the accumulator goes
-// through a per-role epilogue.  Operands are read in place, K-major or MN-major:
-//   forward conv        C[pixel][co] = im2col(act)[pixel][(tap, ci)] W[co][(tap, ci)]^T   (A gathered)
-//   data gradient       one GEMM per output-pixel parity class (py, px) of the stride-2 convolution:
-//                       the input pixel (2Y + py, 2X + px) receives only the taps with ky = 1 (py = 0) or
-//                       ky in {0, 2} (py = 1), and likewise in x, so
-//                       dX_class[(b, Y, X)][ci] = sum over the class's taps and co of
-//                       dY[(b, y(Y, ky), x(X, kx))][co] W[co][ky][kx][ci] -- no col2im
-//   weight gradient     dW[(tap, ci)][co] = sum over pixels of im2col(act)[pixel][(tap, ci)] dY[pixel][co],
-//                       both operands MN-major (channel-contiguous), split over pixels
-//   dense layer         feat W1^T (split K), its weight and data gradients with MN-major operands.
-// Epilogues fuse what surrounds each GEMM: bias and ReLU with the BF16 rounding (forward), the ReLU mask
-// of the layer below with the BF16 rounding of its gradient and per-CTA column sums for its bias
-// gradient (data gradient), transposed partial stores (weight gradients).  The first convolution has a
-// single input channel (K = 9) and runs on the SIMT pipes with the same rounded operands.
+// apply anyway), its sign is the ReLU mask of the backward.  Convolutions 1 to 3 are in cnn_conv.cu; the first one
+// has a single input channel (K = 9) and runs on the SIMT pipes with the same rounded operands.  The dense layer's
+// three GEMMs are launches of one kernel template: 128 threads per CTA, looping over 128-row tiles of C; the four
+// warps fill a ring of 2-4 stages of 64-deep K slices of A and B with 16-byte cp.async copies (zero-filled where an
+// operand is padding), one thread issues the four 128 x BN x 16 MMAs of a slice and commits them to the slice's
+// mbarrier, and the accumulator goes through a per-role epilogue: feat W1^T (split K), the weight gradient
+// (transposed stores) and the data gradient (the last convolution's ReLU mask, its BF16 rounding and per-CTA column
+// sums for its bias gradient), the latter two with MN-major operands.
 // Every mbarrier wait is bounded; a K-loop wait that gives up sets *status and the CTA drains its own
 // MMAs (default bound) before it frees its tensor memory.
 #include <cuda_bf16.h>
@@ -88,106 +78,10 @@ struct PlainMN {  // X[mn][k] = p[k * ld + mn]
   __device__ int zsplit() const { return blockIdx.z; }
 };
 
-// Implicit im2col of a 3 x 3, stride-2, padding-1 convolution over an NHWC input H x W x C (powers of
-// two, C >= 8): row p = output pixel (b, y, x), column (tap, c) = in[b][2y + ky - 1][2x + kx - 1][c].
-struct ConvGeomB {
-  const bf16* act;
-  int H, lwo, lc, rows, cols;  // input height (= width); log2 output width; log2 C; pixels; 9 C
-  __device__ const bf16* at(int p, int kk) const {
-    if (p >= rows || kk >= cols) return nullptr;
-    const int tap = kk >> lc, c = kk & ((1 << lc) - 1), ky = tap / 3, kx = tap - 3 * ky;
-    const int x = p & ((1 << lwo) - 1), y = (p >> lwo) & ((1 << lwo) - 1), b = p >> (2 * lwo);
-    const int iy = 2 * y + ky - 1, ix = 2 * x + kx - 1;
-    if (iy < 0 || iy >= H || ix < 0 || ix >= H) return nullptr;
-    return act + ((((size_t)b * H + iy) * H + ix) << lc) + c;
-  }
-};
-struct ConvK {  // A = im2col, rows = output pixels, reduction = (tap, c)
-  ConvGeomB g;
-  __device__ const bf16* kchunk(int row, int k) const { return g.at(row, k); }
-  __device__ int kdim(int K) const { return K; }
-  __device__ int zsplit() const { return blockIdx.z; }
-};
-struct ConvMN {  // A = im2col^T, rows = (tap, c), reduction = output pixels
-  ConvGeomB g;
-  __device__ const bf16* mnchunk(int mn, int k) const { return g.at(k, mn); }
-  __device__ int kdim(int K) const { return K; }
-  __device__ int zsplit() const { return blockIdx.z; }
-};
-
-// Taps (ky, kx) that reach input pixels of parity class z = 2 py + px, and the offset of the class's
-// weight block (in units of N C) in the class-ordered transposed weights.
-__device__ __forceinline__ int class_taps(int z) { return (z == 0) ? 1 : (z == 3 ? 4 : 2); }
-__device__ __forceinline__ int class_off(int z) { return z == 0 ? 0 : (z == 1 ? 1 : (z == 2 ? 3 : 5)); }
-__host__ __device__ __forceinline__ void class_tap(int z, int t, int& ky, int& kx) {
-  const int py = z >> 1, px = z & 1;
-  const int nx = px ? 2 : 1;
-  const int ty = t / nx, tx = t - ty * nx;
-  ky = py ? 2 * ty : 1;
-  kx = px ? 2 * tx : 1;
-}
-
-// A of the data-gradient GEMM of class z = blockIdx.z: row (b, Y, X) of the class grid (Ho x Ho, the
-// output size of the convolution), reduction (t, co) over the class's taps and the N output channels:
-// dY[b][y][x][co] with 2y + ky - 1 = 2Y + py, 2x + kx - 1 = 2X + px.
-struct ParityK {
-  const bf16* dy;
-  int lho, ln, rows;  // log2 Ho; log2 N; rows = B Ho Ho
-  __device__ const bf16* kchunk(int row, int k) const {
-    if (row >= rows) return nullptr;
-    const int z = blockIdx.z, t = k >> ln, co = k & ((1 << ln) - 1);
-    int ky, kx;
-    class_tap(z, t, ky, kx);
-    const int Ho = 1 << lho;
-    const int X = row & (Ho - 1), Y = (row >> lho) & (Ho - 1), b = row >> (2 * lho);
-    const int y = (2 * Y + (z >> 1) + 1 - ky) >> 1, x = (2 * X + (z & 1) + 1 - kx) >> 1;
-    if (y >= Ho || x >= Ho) return nullptr;
-    return dy + ((((((size_t)b << lho) + y) << lho) + x) << ln) + co;
-  }
-  __device__ int kdim(int) const { return class_taps(blockIdx.z) << ln; }
-  __device__ int zsplit() const { return 0; }  // blockIdx.z is the class, not a split
-};
-
-// B of the data-gradient GEMM: the class's weights transposed, wt[class block][ci][(t, co)].
-struct ClassWt {
-  const bf16* wt;
-  int ln, C;  // log2 N (output channels of the convolution), C input channels (rows)
-  __device__ const bf16* kchunk(int row, int k) const {
-    if (row >= C) return nullptr;
-    const int z = blockIdx.z, kc = class_taps(z) << ln;
-    return wt + ((size_t)class_off(z) << ln) * C + (size_t)row * kc + k;
-  }
-  __device__ int kdim(int K) const { return K; }
-};
-
 // ---- epilogues ---------------------------------------------------------------------------------------
 // apply(row, col0, v[16], acc): the accumulator's row `row`, columns [col0, col0 + 16) of the CTA's tile
 // (global indices); acc is a per-thread running value; finish(...) runs once per thread after all
 // columns, with the CTA's shared scratch (all threads call it).
-
-// BF16 rows (+ bias, ReLU): out[(row / group) * gpitch + (row % group) * rpitch + col].
-struct EpiBf16 {
-  bf16* out;
-  const float* bias;
-  int relu, rows, group, gpitch, rpitch;
-  __device__ void apply(int row, int col0, float v[16], float&, float*) const {
-    if (row >= rows) return;
-    uint32_t w[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float a = v[2 * j] + bias[col0 + 2 * j], b = v[2 * j + 1] + bias[col0 + 2 * j + 1];
-      if (relu) {
-        a = fmaxf(a, 0.f);
-        b = fmaxf(b, 0.f);
-      }
-      w[j] = pack2(a, b);
-    }
-    uint4* d = reinterpret_cast<uint4*>(out + (size_t)(row / group) * gpitch + (size_t)(row % group) * rpitch + col0);
-    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    d[1] = make_uint4(w[4], w[5], w[6], w[7]);
-  }
-  __device__ void finish(int, float, float*, int, int, int) const {}
-};
 
 // FP32 rows of split z: part[z * zstride + row * ld + col].
 struct EpiF32 {
@@ -235,52 +129,6 @@ __device__ __forceinline__ float warp_sum16(float v[16], int lane) {
 __device__ __forceinline__ int sum16_col(int lane) {
   return 8 * ((lane >> 4) & 1) + 4 * ((lane >> 3) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1);
 }
-
-// Data gradient of class z: row (b, Y, X) is input pixel (b, 2Y + py, 2X + px) of a layer with C = BN
-// channels and H x H pixels; dY_in = dX * [act > 0] (act: that layer's post-ReLU output), stored in BF16
-// at the NHWC index; the masked FP32 values are summed per column over the CTA's rows into
-// colpart[z * n_mt + mt][col] (bias gradient of that layer; mt the row tile).
-template <int BN>
-struct EpiDx {
-  bf16* dy_out;
-  const bf16* act;
-  float* colpart;
-  int lho, H, rows;
-  __device__ void apply(int row, int col0, float v[16], float&, float* scratch) const {
-    const int z = blockIdx.z;
-    if (row < rows) {
-      const int Ho = 1 << lho;
-      const int X = row & (Ho - 1), Y = (row >> lho) & (Ho - 1), b = row >> (2 * lho);
-      const size_t idx = (((size_t)b * H + 2 * Y + (z >> 1)) * H + 2 * X + (z & 1)) * BN + col0;
-      const uint4* a = reinterpret_cast<const uint4*>(act + idx);
-      float m[16];
-      unpack8(a[0], m);
-      unpack8(a[1], m + 8);
-      uint32_t w[8];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = m[j] > 0.f ? v[j] : 0.f;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) w[j] = pack2(v[2 * j], v[2 * j + 1]);
-      uint4* d = reinterpret_cast<uint4*>(dy_out + idx);
-      d[0] = make_uint4(w[0], w[1], w[2], w[3]);
-      d[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = 0.f;
-    }
-    // column sums over the warp's 32 rows, into the shared scratch [warp][BN] (written in finish order)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float s = warp_sum16(v, lane);
-    if ((lane & 1) == 0) scratch[warp * BN + col0 - blockIdx.y * BN + sum16_col(lane)] = s;
-  }
-  __device__ void finish(int, float, float* scratch, int tid, int mt, int n_mt) const {
-    __syncthreads();
-    if (tid < BN) {
-      const float s = scratch[tid] + scratch[BN + tid] + scratch[2 * BN + tid] + scratch[3 * BN + tid];
-      colpart[((size_t)blockIdx.z * n_mt + mt) * BN + tid] = s;
-    }
-  }
-};
 
 // Gradient of the dense layer's input, rows b (batch entry) and columns f (feature, blockIdx.y selects
 // 128 of them, i.e. one pixel's 128 channels of the last convolution):
@@ -634,9 +482,10 @@ __global__ void __launch_bounds__(256) k_colreduce_once(const float* __restrict_
 
 // out[i] = sum over z of part[z * n + i] (+ bias[i % nb] and ReLU when bias != nullptr), in a fixed order:
 // 32 outputs per block, warp w adding the splits z = w, w + 8, ... in order (coalesced over the outputs),
-// then the eight warp sums added in warp order.
+// then the eight warp sums added in warp order.  NaN where a kernel of this pass gave up waiting (*status).
 __global__ void __launch_bounds__(256) k_sum_z(const float* __restrict__ part, int Z, long long n,
-                                               const float* __restrict__ bias, int nb, float* __restrict__ out) {
+                                               const float* __restrict__ bias, int nb, float* __restrict__ out,
+                                               const unsigned* status) {
   __shared__ float red[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long i = (long long)blockIdx.x * 32 + lane;
@@ -650,15 +499,18 @@ __global__ void __launch_bounds__(256) k_sum_z(const float* __restrict__ part, i
 #pragma unroll
     for (int w = 1; w < 8; ++w) t += red[w][lane];
     if (bias) t = fmaxf(t + bias[i % nb], 0.f);
+    if (status && *status) t = __int_as_float(0x7fffffff);
     out[i] = t;
   }
 }
 
 // All of a forward's weight conversions to BF16 in one launch: job k covers the elements [start[k], start[k + 1])
 // of a grid-stride loop.  Kind 0, rows: out[r][c] = BF16 of in[r][c] for c < b, 0 for b <= c < c_pitch
-// (a rows, row pitch c).  Kind 1, the class-ordered transposed weights of a convolution with N = a output
-// and C = b input channels: out[class block z][ci][(t, co)] = BF16 of w[co][ky_t][kx_t][ci] for the
-// class's taps t.  Kind 2: out[e] = BF16 of in[e].
+// (a rows, row pitch c).  Kind 1, the transposed weights of a convolution with N = a output and C = b input
+// channels for its data gradient (Dx in cnn_conv.cu): rows of 64 output channels, in blocks of CC = min(C, 64) input
+// channels, for each CC of the C the blocks of the four shifts (dy, dx) (for each 64 of the N): 4, 2, 2 and 1
+// parity classes, the class (py, px) of a shift taking the tap ky = py ? 2 - 2 dy : 1, kx = px ? 2 - 2 dx : 1.
+// *status is set to zero for the kernels that follow.
 struct BfJob {
   const float* in;
   bf16* out;
@@ -669,7 +521,8 @@ struct BfJobs {
   long long start[9];
   int count;
 };
-__global__ void __launch_bounds__(256) k_to_bf16_jobs(const __grid_constant__ BfJobs J) {
+__global__ void __launch_bounds__(256) k_to_bf16_jobs(const __grid_constant__ BfJobs J, unsigned* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0u;
   const long long total = J.start[J.count];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     int k = 0;
@@ -680,17 +533,15 @@ __global__ void __launch_bounds__(256) k_to_bf16_jobs(const __grid_constant__ Bf
     if (jb.kind == 0) {
       const int r = (int)(e / jb.c), c = (int)(e - (long long)r * jb.c);
       x = c < jb.b ? jb.in[(size_t)r * jb.b + c] : 0.f;
-    } else if (jb.kind == 1) {
-      const long long NC = (long long)jb.a * jb.b;
-      const int z = e < NC ? 0 : (e < 3 * NC ? 1 : (e < 5 * NC ? 2 : 3));
-      const long long local = e - (long long)class_off(z) * NC;
-      const int kc = class_taps(z) * jb.a;
-      const int ci = (int)(local / kc), rem = (int)(local - (long long)ci * kc), t = rem / jb.a, co = rem - t * jb.a;
-      int ky, kx;
-      class_tap(z, t, ky, kx);
-      x = jb.in[((size_t)co * 9 + ky * 3 + kx) * jb.b + ci];
     } else {
-      x = jb.in[e];
+      const int CC = min(jb.b, 64), H = jb.a / 64, row = (int)(e >> 6), chunk = row / (9 * H * CC);
+      const int blk = row / CC - chunk * 9 * H, ci = chunk * CC + row % CC;
+      const int shift = blk < 4 * H ? 0 : blk / (2 * H) - 1;  // blocks [0, 4H), [4H, 6H), [6H, 8H), [8H, 9H)
+      const int nb = shift == 0 ? 4 : (shift == 3 ? 1 : 2), k2 = blk - (shift == 0 ? 0 : 2 + 2 * shift) * H;
+      const int half = k2 / nb, pos = k2 % nb + (shift >= 2);
+      const int cls = pos == 0 ? 1 : (pos == 1 ? 3 : (pos == 2 ? 2 : 0));
+      const int ky = (cls >> 1) ? 2 - 2 * (shift >> 1) : 1, kx = (cls & 1) ? 2 - 2 * (shift & 1) : 1;
+      x = jb.in[((size_t)(half * 64 + (int)(e & 63)) * 9 + ky * 3 + kx) * jb.b + ci];
     }
     jb.out[e] = __float2bfloat16_rn(x);
   }
@@ -737,17 +588,9 @@ cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy,
     if (e__ != cudaSuccess) return e__;   \
   } while (0)
 
-// Splits of a pixel-reduction weight gradient: about two CTAs per SM over the row tiles, at least four
-// 64-pixel slices per split, partials within the buffer.
 constexpr int kConv0Ctas = 4 * 152;  // k_conv0_dw: four CTAs per SM (its register limit)
 constexpr int kColTickets = 64;      // colreduce ticket counters (column groups of 32)
 
-int dw_splits(int tiles, long long pixels, long long part_floats, long long tile_floats) {
-  long long z = (2LL * 152 + tiles - 1) / tiles;
-  z = std::min(z, std::max(1LL, pixels / 256));
-  z = std::min(z, std::max(1LL, part_floats / tile_floats));
-  return (int)std::max(1LL, z);
-}
 int chunk_of(long long n, int z) { return (int)(((n + z - 1) / z + kBK - 1) / kBK * kBK); }
 
 // out[c] = sum over r < R of in[r * ld + c] in a fixed order: row chunks of 64 summed into scratch by
@@ -803,13 +646,14 @@ size_t cnn_tc_layout(void* base, int B, CnnTc* t) {
   w.colpart_floats = std::max<long long>({1024LL * B, 8192LL * ((B + 127) / 128), (long long)kConv0Ctas * 288});
   w.colpart = (float*)take((size_t)w.colpart_floats * 4);
   w.tickets = (unsigned*)take(kColTickets * sizeof(unsigned));
+  w.status = (unsigned*)take(sizeof(unsigned));
   if (t) *t = w;
   return off;
 }
 
 cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs, int B, const CnnTc& t, float* h,
                            cudaStream_t st) {
-  // BF16 copies of the weights, row-major (forward) and class-ordered transposed (data gradient): one
+  // BF16 copies of the weights, row-major (forward) and transposed (data gradient): one
   // launch (the first convolution rounds the input images itself and stores their BF16 copy)
   BfJobs J{};
   long long at = 0;
@@ -825,26 +669,15 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
   }
   add(net.w1, (bf16*)t.w1b, 0, kHid, kFeat + 2, kFeatPitch, (long long)kHid * kFeatPitch);
   J.start[J.count] = at;
-  k_to_bf16_jobs<<<grid_of(at), 256, 0, st>>>(J);
+  k_to_bf16_jobs<<<grid_of(at), 256, 0, st>>>(J, t.status);
   const int npix0 = B * 4096;
   k_conv0_fwd<<<(npix0 + 255) / 256, 256, 0, st>>>(img, net.w[0], net.b[0], npix0, (bf16*)t.act[0], (bf16*)t.imgb);
   note_launches(2);
   const void* any = t.wb[1];
   for (int l = 1; l < 4; ++l) {
-    const int H = kEdge[l], lwo = l == 1 ? 5 : (l == 2 ? 4 : 3), lc = l == 1 ? 5 : (l == 2 ? 6 : 7);
-    const int rows = B * kEdge[l + 1] * kEdge[l + 1], N = kCh[l + 1], Kl = 9 * kCh[l];
-    const ConvK A{ConvGeomB{(const bf16*)t.act[l - 1], H, lwo, lc, rows, Kl}};
-    const PlainK Bw{(const bf16*)t.wb[l], Kl, N};
-    if (l == 1) {
-      const EpiBf16 ep{(bf16*)t.act[1], net.b[1], 1, rows, 1 << 30, 0, N};
-      TC_TRY((gemm<64, 2, false, false>(A, Bw, ep, rows, Kl, 1, 1, Kl, any, st)));
-    } else if (l == 2) {
-      const EpiBf16 ep{(bf16*)t.act[2], net.b[2], 1, rows, 1 << 30, 0, N};
-      TC_TRY((gemm<128, 3, false, false>(A, Bw, ep, rows, Kl, 1, 1, Kl, any, st)));
-    } else {  // the last convolution writes the dense layer's feature rows ((y, x, c) order, pitch 8200)
-      const EpiBf16 ep{(bf16*)t.feat, net.b[3], 1, rows, 64, kFeatPitch, N};
-      TC_TRY((gemm<128, 4, false, false>(A, Bw, ep, rows, Kl, 1, 1, Kl, any, st)));
-    }
+    // the last convolution writes the dense layer's feature rows ((y, x, c) order, pitch 8200)
+    const long long pitch = l == 3 ? kFeatPitch : (long long)kEdge[l + 1] * kEdge[l + 1] * kCh[l + 1];
+    TC_TRY(cnn_conv_forward(l, t.act[l - 1], t.wb[l], net.b[l], B, l == 3 ? t.feat : t.act[l], pitch, t.status, st));
   }
   k_feat_tail<<<(B * (kFeatPitch - kFeat) + 255) / 256, 256, 0, st>>>((bf16*)t.feat, cs, B);
   note_launches(1);
@@ -853,7 +686,7 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
   const EpiF32 ep{t.part, (long long)B * kHid, B, kHid};
   TC_TRY((gemm<128, 4, false, false>(PlainK{(const bf16*)t.feat, kFeatPitch, B}, PlainK{(const bf16*)t.w1b, kFeatPitch, kHid},
                                   ep, B, kFeatPitch, 1, Z, kc, any, st)));
-  k_sum_z<<<(unsigned)(((long long)B * kHid + 31) / 32), 256, 0, st>>>(t.part, Z, (long long)B * kHid, net.b1, kHid, h);
+  k_sum_z<<<(unsigned)(((long long)B * kHid + 31) / 32), 256, 0, st>>>(t.part, Z, (long long)B * kHid, net.b1, kHid, h, t.status);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -874,40 +707,21 @@ cudaError_t cnn_tc_backward(int B, const CnnTc& t, const float* dh, const CnnGra
                                     kHid, any, st)));
   TC_TRY(colreduce(t.colpart, (kFeat / 128) * nmt, 128, 128, g.b[3], t.part, t.tickets, st));
   // convolutions 3, 2, 1: weight gradient (split over pixels), then the data gradient of the layer below
-  const bf16* dyl = (const bf16*)t.dy3;
+  const uint16_t* dyl = t.dy3;
   for (int l = 3; l >= 1; --l) {
-    const int H = kEdge[l], lwo = l == 1 ? 5 : (l == 2 ? 4 : 3), lc = l == 1 ? 5 : (l == 2 ? 6 : 7);
-    const int ln = l == 1 ? 6 : 7;  // log2 N_l
-    const int rows = B * kEdge[l + 1] * kEdge[l + 1], N = kCh[l + 1], Kl = 9 * kCh[l], C = kCh[l];
-    const ConvGeomB geo{(const bf16*)t.act[l - 1], H, lwo, lc, rows, Kl};
-    const int tiles = (Kl + kBM - 1) / kBM;
-    const int Z = dw_splits(tiles, rows, t.part_floats, (long long)N * Kl);
-    const int kc = chunk_of(rows, Z);
-    const EpiF32T epw{t.part, (long long)N * Kl, Kl, Kl};
-    if (N == 64)
-      TC_TRY((gemm<64, 3, true, true>(ConvMN{geo}, PlainMN{dyl, N, N}, epw, Kl, rows, 1, Z, kc, any, st)));
-    else
-      TC_TRY((gemm<128, 4, true, true>(ConvMN{geo}, PlainMN{dyl, N, N}, epw, Kl, rows, 1, Z, kc, any, st)));
-    k_sum_z<<<(unsigned)(((long long)N * Kl + 31) / 32), 256, 0, st>>>(t.part, Z, (long long)N * Kl, nullptr, 1, g.w[l]);
+    const long long n = 9LL * kCh[l] * kCh[l + 1];
+    const int Z = cnn_conv_dw_splits(l, B, t.part_floats);
+    TC_TRY(cnn_conv_dw(l, t.act[l - 1], dyl, B, t.part, Z, t.status, st));
+    k_sum_z<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(t.part, Z, n, nullptr, 1, g.w[l], t.status);
     note_launches(1);
-    // data gradient, four parity classes in one launch; output dY of conv l - 1 and its bias partials
-    bf16* dyo = (bf16*)(l == 2 ? t.dy[1] : t.dy[0]);
-    const ParityK A{dyl, lwo, ln, rows};
-    const ClassWt Bw{(const bf16*)t.wt[l], ln, C};
-    if (C == 128)
-      TC_TRY((gemm<128, 3, false, false>(A, Bw, EpiDx<128>{dyo, (const bf16*)t.act[l - 1], t.colpart, lwo, H, rows}, rows,
-                                      9 * N, 1, 4, 1 << 30, any, st)));
-    else if (C == 64)
-      TC_TRY((gemm<64, 2, false, false>(A, Bw, EpiDx<64>{dyo, (const bf16*)t.act[l - 1], t.colpart, lwo, H, rows}, rows,
-                                     9 * N, 1, 4, 1 << 30, any, st)));
-    else
-      TC_TRY((gemm<32, 2, false, false>(A, Bw, EpiDx<32>{dyo, (const bf16*)t.act[l - 1], t.colpart, lwo, H, rows}, rows,
-                                     9 * N, 1, 4, 1 << 30, any, st)));
-    TC_TRY(colreduce(t.colpart, 4 * ((rows + kBM - 1) / kBM), C, C, g.b[l - 1], t.part, t.tickets, st));
+    // output dY of convolution l - 1 and its bias partials, a row per CTA
+    uint16_t* dyo = l == 2 ? t.dy[1] : t.dy[0];
+    TC_TRY(cnn_conv_dx(l, dyl, t.wt[l], t.act[l - 1], B, dyo, t.colpart, t.status, st));
+    TC_TRY(colreduce(t.colpart, cnn_conv_dx_rows(l, B), kCh[l], kCh[l], g.b[l - 1], t.part, t.tickets, st));
     dyl = dyo;
   }
   // the first convolution's weight gradient on the SIMT pipes
-  TC_TRY(conv0_dw(dyl, (const bf16*)t.imgb, B, t.colpart, t.part, t.tickets, g.w[0], st));
+  TC_TRY(conv0_dw((const bf16*)dyl, (const bf16*)t.imgb, B, t.colpart, t.part, t.tickets, g.w[0], st));
   return cudaGetLastError();
 }
 
@@ -922,7 +736,7 @@ cudaError_t cnn_conv0_dw_f32(const float* dy, const float* img, int B, const Cnn
 }
 
 cudaError_t cnn_sum_splits(const float* part, int Z, long long n, const float* bias, int nb, float* out, cudaStream_t st) {
-  k_sum_z<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(part, Z, n, bias, nb, out);
+  k_sum_z<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(part, Z, n, bias, nb, out, nullptr);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -145,6 +145,7 @@ struct CnnTc {
   float *part, *colpart;
   long long part_floats, colpart_floats;
   unsigned* tickets;  // counters of the single-launch column reductions (zeroed by cnn_tc_backward)
+  unsigned* status;   // zeroed by cnn_tc_forward; set by a convolution kernel that gave up waiting
 };
 // Bytes of the buffers for batch B (base == nullptr: size only), 256-byte aligned.
 size_t cnn_tc_layout(void* base, int B, CnnTc* t);
@@ -162,6 +163,20 @@ cudaError_t cnn_colsum(const float* dY, int M, int N, const CnnTc& t, float* out
 // (t: scratch), and out[i] = sum over z of part[z n + i] (+ bias[i % nb] and ReLU when bias is given).
 cudaError_t cnn_conv0_dw_f32(const float* dy, const float* img, int B, const CnnTc& t, float* out, cudaStream_t st);
 cudaError_t cnn_sum_splits(const float* part, int Z, long long n, const float* bias, int nb, float* out, cudaStream_t st);
+
+// cnn_conv.cu: convolutions l = 1 to 3 of the tensor-core path.  Forward: out [B][pixels][N] (BF16, images `pitch`
+// elements apart) = ReLU(conv(act, w [N][9 C]) + bias).
+cudaError_t cnn_conv_forward(int l, const uint16_t* act, const uint16_t* w, const float* bias, int B, uint16_t* out,
+                             long long pitch, unsigned* status, cudaStream_t st);
+// dx = (gradient of the convolution's input) * [act > 0] in BF16, wt as k_to_bf16_jobs lays it out; the masked FP32
+// values summed over pixels into cnn_conv_dx_rows partial rows colpart[row][C].
+int cnn_conv_dx_rows(int l, int B);
+cudaError_t cnn_conv_dx(int l, const uint16_t* dy, const uint16_t* wt, const uint16_t* act, int B, uint16_t* dx,
+                        float* colpart, unsigned* status, cudaStream_t st);
+// Weight gradient [N][9 C] in Z partial sums over the pixels (FP32).
+int cnn_conv_dw_splits(int l, int B, long long part_floats);
+cudaError_t cnn_conv_dw(int l, const uint16_t* act, const uint16_t* dy, int B, float* part, int Z, unsigned* status,
+                        cudaStream_t st);
 
 // cnn_f32.cu: the same network in FP32 on the SIMT pipes (buffers of one batch size, all FP32).
 struct CnnF32 {
