@@ -335,54 +335,16 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
 
 // ---- SIMT kernels and small steps --------------------------------------------------------------------
 
-// First convolution (1 -> 32 channels, 128^2 -> 64^2): act0[p][co] = relu(b[co] + sum over taps of
-// r(w[co][tap]) r(img(tap))), r = BF16 rounding, img the FP32 input; one thread per output pixel, 32
-// channels stored as four 16-byte BF16 chunks; the rounded input is also stored (imgb) for the backward.
-__global__ void __launch_bounds__(256) k_conv0_fwd(const float* __restrict__ img, const float* __restrict__ w,
-                                                   const float* __restrict__ bias, int npix, bf16* __restrict__ out,
-                                                   bf16* __restrict__ imgb) {
-  __shared__ float sw[32 * 9], sb[32];
-  for (int i = threadIdx.x; i < 32 * 9; i += blockDim.x) sw[i] = bf16r(w[i]);
-  if (threadIdx.x < 32) sb[threadIdx.x] = bias[threadIdx.x];
-  __syncthreads();
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= npix) return;
-  const int x = p & 63, y = (p >> 6) & 63, b = p >> 12;
-  float xin[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    const int iy = 2 * y + t / 3 - 1, ix = 2 * x + t % 3 - 1;
-    xin[t] = (iy >= 0 && iy < 128 && ix >= 0 && ix < 128) ? bf16r(img[((size_t)b * 128 + iy) * 128 + ix]) : 0.f;
-  }
-  // the BF16 input the weight gradient reads: this pixel writes input pixels (2y + dy, 2x + dx), dy, dx in
-  // {0, 1} (its taps 4, 5, 7, 8), so every input pixel is written exactly once
-  {
-    uint32_t* row0 = reinterpret_cast<uint32_t*>(imgb + ((size_t)b * 128 + 2 * y) * 128 + 2 * x);
-    row0[0] = pack2(xin[4], xin[5]);
-    row0[64] = pack2(xin[7], xin[8]);  // the next row: 128 BF16 = 64 words further
-  }
-  uint4* d = reinterpret_cast<uint4*>(out + (size_t)p * 32);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float o[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int co = 8 * q + j;
-      float a = sb[co];
-#pragma unroll
-      for (int t = 0; t < 9; ++t) a = fmaf(sw[co * 9 + t], xin[t], a);
-      o[j] = fmaxf(a, 0.f);
-    }
-    d[q] = make_uint4(pack2(o[0], o[1]), pack2(o[2], o[3]), pack2(o[4], o[5]), pack2(o[6], o[7]));
-  }
-}
+// ---- first convolution (1 -> 32 channels, 128^2 -> 64^2) ---------------------------------------------
+// Both directions work on bands of kBandRows output rows of one image, whose input rows lie in shared memory as
+// FP32 (columns -1 to 127; zeros outside the image).  Four lanes share an output pixel, 8 channels each: their
+// weights (or their sums of the weight gradient) stay in 72 registers, a pixel's 9 inputs are broadcast reads, and
+// a warp's 16-byte accesses of act0 and dY0 cover eight whole pixels in a row.
+// What bounds them: 288 FMAs a pixel, then HBM.  With a thread per pixel the forward read a weight from shared
+// memory for every FMA and stored 16 bytes per lane 64 bytes apart, and the gradient loaded nine inputs from global
+// memory for 36 FMAs.  Batch 256: forward 33.6 -> 22.2 us, weight gradient 52.5 -> 23.3 us.
+constexpr int kBandRows = 8, kBands = 64 / kBandRows, kBandIn = 2 * kBandRows + 1, kBandPitch = 132;
 
-// Weight gradient of the first convolution: part[block][co * 9 + tap] = sum over the block's pixels of
-// dY0[p][co] img(tap), both of type T (BF16, or FP32 for the FP32 mode).  Thread t owns the channels
-// 4 (t & 7) ... + 3 and the pixel stream t >> 3 (32 streams per block, grid-stride over the pixels, two
-// pixels per step with all their loads issued first); its 36 products per pixel accumulate in registers,
-// and the block's 32 streams are added in a fixed order through shared memory.  A GEMM tile of 64 x 64 for
-// this 32 x 9 result works on padding: in FP32 and batch 64, 578 us as a GEMM, 18 us here.
 __device__ __forceinline__ void load4(const bf16* p, float d[4]) {
   const uint2 u = *reinterpret_cast<const uint2*>(p);
   d[0] = __uint_as_float(u.x << 16);
@@ -397,43 +359,191 @@ __device__ __forceinline__ void load4(const float* p, float d[4]) {
 __device__ __forceinline__ float to_float(bf16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float to_float(float x) { return x; }
 
+// A band's share of a thread (of 256): input rows 2 y0 - 1 ... 2 y0 + 15 of image b, 4 columns at a time.
+struct BandPart {
+  float v[3][4];
+};
 template <typename T>
-__global__ void __launch_bounds__(256, 4) k_conv0_dw(const T* __restrict__ dy, const T* __restrict__ img, int npix,
-                                                     float* __restrict__ part) {
-  __shared__ float red[32][289];
-  const int cg = threadIdx.x & 7, sid = threadIdx.x >> 3;
-  float acc[4][9];
+__device__ __forceinline__ void fetch_band(const T* __restrict__ img, bool wide, int b, int y0, BandPart& o) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int k = 0; k < 3; ++k) {
+    const int i = threadIdx.x + 256 * k, iy = 2 * y0 - 1 + (i >> 5);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o.v[k][e] = 0.f;
+    if (i >= kBandIn * 32 || iy < 0) continue;
+    const T* p = img + ((size_t)b * 128 + iy) * 128 + (i & 31) * 4;
+    if (wide) {
+      load4(p, o.v[k]);
+    } else {  // the caller's images need only be aligned to their elements
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o.v[k][e] = to_float(p[e]);
+    }
+  }
+}
+// ... into s[row][4 + column] (s[row][3] = column -1 = 0); with ROUND rounded to BF16, and rows 2 y0 ... also stored
+// to imgb (every row by one band).
+template <bool ROUND>
+__device__ __forceinline__ void put_band(BandPart& o, int b, int y0, float (*s)[kBandPitch], bf16* imgb) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int i = threadIdx.x + 256 * k, r = i >> 5, c = (i & 31) * 4;
+    if (i >= kBandIn * 32) continue;
+    float* v = o.v[k];
+    if (ROUND) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = bf16r(v[e]);
+      if (r > 0)
+        *reinterpret_cast<uint2*>(imgb + ((size_t)b * 128 + 2 * y0 - 1 + r) * 128 + c) =
+            make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
+    }
+    *reinterpret_cast<float4*>(&s[r][4 + c]) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  if (threadIdx.x < kBandIn) s[threadIdx.x][3] = 0.f;
+}
+// The 9 inputs of output pixel (row r of the band, x).
+__device__ __forceinline__ void taps9(const float (*s)[kBandPitch], int r, int x, float v[9]) {
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky) {
+    v[3 * ky] = s[2 * r + ky][3 + 2 * x];
+    const float2 u = *reinterpret_cast<const float2*>(&s[2 * r + ky][4 + 2 * x]);
+    v[3 * ky + 1] = u.x;
+    v[3 * ky + 2] = u.y;
+  }
+}
+
+// act0[p][co] = relu(b[co] + sum over taps of r(w[co][tap]) r(img(tap))), r = BF16 rounding, stored in BF16 with the
+// rounded input (imgb) for the backward.  Blocks stride over the n_bands bands, the next one's inputs on the way
+// during the sums of the last.
+__global__ void __launch_bounds__(256, 2) k_conv0_fwd(const float* __restrict__ img, const float* __restrict__ w,
+                                                      const float* __restrict__ bias, int n_bands, bf16* __restrict__ out,
+                                                      bf16* __restrict__ imgb) {
+  __shared__ __align__(16) float s[2][kBandIn][kBandPitch];
+  const int q = threadIdx.x & 3, x = threadIdx.x >> 2;
+  const bool wide = ((uintptr_t)img & 15) == 0;
+  int band = blockIdx.x;
+  BandPart part;
+  fetch_band(img, wide, band / kBands, band % kBands * kBandRows, part);
+  float wr[8][9], br[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    br[j] = bias[q * 8 + j];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) wr[j][t] = bf16r(w[(q * 8 + j) * 9 + t]);
+  }
+  for (int buf = 0; band < n_bands; buf ^= 1) {
+    const int b = band / kBands, y0 = band % kBands * kBandRows;
+    put_band<true>(part, b, y0, s[buf], imgb);
+    __syncthreads();  // one a band: a buffer's readers have passed the next band's barrier before it is refilled
+    band += gridDim.x;
+    if (band < n_bands) fetch_band(img, wide, band / kBands, band % kBands * kBandRows, part);
+#pragma unroll 1
+    for (int r = 0; r < kBandRows; ++r) {
+      float v[9], o[8];
+      taps9(s[buf], r, x, v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float a = br[j];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) a = fmaf(wr[j][t], v[t], a);
+        o[j] = fmaxf(a, 0.f);
+      }
+      *reinterpret_cast<uint4*>(out + (((size_t)b * 64 + y0 + r) * 64 + x) * 32 + q * 8) =
+          make_uint4(pack2(o[0], o[1]), pack2(o[2], o[3]), pack2(o[4], o[5]), pack2(o[6], o[7]));
+    }
+  }
+}
+
+// Weight gradient: part[block][co * 9 + tap] = sum over the block's bands of dY0[p][co] img(tap), both of type T
+// (BF16, or FP32 for the FP32 mode), blocks striding over the n_bands bands.  A thread's column of pixels adds up in
+// its registers; the 64 columns are added at the end in a fixed order.
+template <typename T>
+__global__ void __launch_bounds__(256, 2) k_conv0_dw(const T* __restrict__ dy, const T* __restrict__ img, int n_bands,
+                                                     float* __restrict__ part) {
+  __shared__ __align__(16) float s[kBandIn][kBandPitch];
+  const int q = threadIdx.x & 3, x = threadIdx.x >> 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float acc[8][9];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
     for (int t = 0; t < 9; ++t) acc[j][t] = 0.f;
-  const long long stride = (long long)gridDim.x * 32;
-#pragma unroll 2
-  for (long long p = (long long)blockIdx.x * 32 + sid; p < npix; p += stride) {
-    float d[4];
-    load4(dy + p * 32 + cg * 4, d);
-    const int x = (int)(p & 63), y = (int)((p >> 6) & 63), b = (int)(p >> 12);
-    float xv[9];
+  constexpr int A = sizeof(T) == 2 ? 4 : 2, W = sizeof(T) / 2;  // rows of dY0 fetched ahead, 16-byte words of 8 channels
+  for (int band = blockIdx.x; band < n_bands; band += gridDim.x) {
+    const int b = band / kBands, y0 = band % kBands * kBandRows;
+    const T* d0 = dy + (((size_t)b * 64 + y0) * 64 + x) * 32 + q * 8;
+    uint4 cur[A][W], next[A][W];
+    auto fetch = [&](uint4 (*u)[W], int r) {
+#pragma unroll
+      for (int k = 0; k < A; ++k)
+#pragma unroll
+        for (int e = 0; e < W; ++e) u[k][e] = __ldg(reinterpret_cast<const uint4*>(d0 + (size_t)(r + k) * 64 * 32) + e);
+    };
+    fetch(cur, 0);
+    BandPart p;
+    fetch_band(img, true, b, y0, p);
+    __syncthreads();
+    put_band<false>(p, b, y0, s, nullptr);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kBandRows; r += A) {
+      if (r + A < kBandRows) fetch(next, r + A);
+#pragma unroll
+      for (int k = 0; k < A; ++k) {
+        float d[8], v[9];
+        if constexpr (W == 1) {
+          unpack8(cur[k][0], d);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            d[4 * e] = __uint_as_float(cur[k][e].x);
+            d[4 * e + 1] = __uint_as_float(cur[k][e].y);
+            d[4 * e + 2] = __uint_as_float(cur[k][e].z);
+            d[4 * e + 3] = __uint_as_float(cur[k][e].w);
+          }
+        }
+        taps9(s, r + k, x, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+          for (int t = 0; t < 9; ++t) acc[j][t] = fmaf(d[j], v[t], acc[j][t]);
+      }
+#pragma unroll
+      for (int k = 0; k < A; ++k)
+#pragma unroll
+        for (int e = 0; e < W; ++e) cur[k][e] = next[k][e];
+    }
+  }
+  __syncthreads();
+  float* red = &s[0][0];  // [warp][288] of four warps at a time (8 x 288 do not fit)
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
-      const int iy = 2 * y + t / 3 - 1, ix = 2 * x + t % 3 - 1;
-      xv[t] = (iy >= 0 && iy < 128 && ix >= 0 && ix < 128) ? to_float(img[((size_t)b * 128 + iy) * 128 + ix]) : 0.f;
+      float a = acc[j][t];
+      a += __shfl_xor_sync(0xffffffffu, a, 4);
+      a += __shfl_xor_sync(0xffffffffu, a, 8);
+      a += __shfl_xor_sync(0xffffffffu, a, 16);
+      acc[j][t] = a;
     }
+  float sum[2] = {0.f, 0.f};
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    if ((warp >> 2) == h && lane < 4) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < 8; ++j)
 #pragma unroll
-      for (int t = 0; t < 9; ++t) acc[j][t] = fmaf(d[j], xv[t], acc[j][t]);
+        for (int t = 0; t < 9; ++t) red[(warp & 3) * 288 + (q * 8 + j) * 9 + t] = acc[j][t];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int o = threadIdx.x + 256 * k;
+      if (o < 288) sum[k] += (red[o] + red[288 + o]) + (red[576 + o] + red[864 + o]);
+    }
+    __syncthreads();
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) red[sid][(cg * 4 + j) * 9 + t] = acc[j][t];
-  __syncthreads();
-  for (int o = threadIdx.x; o < 288; o += blockDim.x) {
-    float sum = 0.f;
-    for (int k = 0; k < 32; ++k) sum += red[k][o];
-    part[(size_t)blockIdx.x * 288 + o] = sum;
-  }
+  for (int k = 0; k < 2; ++k)
+    if (threadIdx.x + 256 * k < 288) part[(size_t)blockIdx.x * 288 + threadIdx.x + 256 * k] = sum[k];
 }
 
 // out[c] = sum over the rows r < R of in[r * ld + c], in one launch: block (x, y) sums rows
@@ -588,7 +698,7 @@ cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy,
     if (e__ != cudaSuccess) return e__;   \
   } while (0)
 
-constexpr int kConv0Ctas = 4 * 152;  // k_conv0_dw: four CTAs per SM (its register limit)
+constexpr int kConv0Ctas = 2 * 152;  // two CTAs per SM (the registers of k_conv0_fwd and _dw)
 constexpr int kColTickets = 64;      // colreduce ticket counters (column groups of 32)
 
 int chunk_of(long long n, int z) { return (int)(((n + z - 1) / z + kBK - 1) / kBK * kBK); }
@@ -606,13 +716,14 @@ cudaError_t colreduce(const float* in, int R, int cols, int ld, float* out, floa
   return cudaGetLastError();
 }
 
-// dW of the first convolution into out (32 x 9): kConv0Ctas partial sums in colpart, then added.
+// dW of the first convolution into out (32 x 9): at most kConv0Ctas partial sums in colpart, then added.
 template <typename T>
 cudaError_t conv0_dw(const T* dy, const T* img, int B, float* colpart, float* scratch, unsigned* tickets, float* out,
                      cudaStream_t st) {
-  k_conv0_dw<T><<<kConv0Ctas, 256, 0, st>>>(dy, img, B * 4096, colpart);
+  const int ctas = std::min(kConv0Ctas, B * kBands);
+  k_conv0_dw<T><<<ctas, 256, 0, st>>>(dy, img, B * kBands, colpart);
   note_launches(1);
-  return colreduce(colpart, kConv0Ctas, 288, 288, out, scratch, tickets, st);
+  return colreduce(colpart, ctas, 288, 288, out, scratch, tickets, st);
 }
 
 }  // namespace
@@ -670,8 +781,8 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
   add(net.w1, (bf16*)t.w1b, 0, kHid, kFeat + 2, kFeatPitch, (long long)kHid * kFeatPitch);
   J.start[J.count] = at;
   k_to_bf16_jobs<<<grid_of(at), 256, 0, st>>>(J, t.status);
-  const int npix0 = B * 4096;
-  k_conv0_fwd<<<(npix0 + 255) / 256, 256, 0, st>>>(img, net.w[0], net.b[0], npix0, (bf16*)t.act[0], (bf16*)t.imgb);
+  k_conv0_fwd<<<std::min(kConv0Ctas, B * kBands), 256, 0, st>>>(img, net.w[0], net.b[0], B * kBands, (bf16*)t.act[0],
+                                                                (bf16*)t.imgb);
   note_launches(2);
   const void* any = t.wb[1];
   for (int l = 1; l < 4; ++l) {

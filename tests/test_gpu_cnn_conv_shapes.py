@@ -28,3 +28,14 @@ def test_forward_and_gradient_at_tile_edges(P, B):  # noqa: F811
         k = int(np.prod(shape))
         assert relL2(g[off:off + k], gref[off:off + k]) < 3e-3, name
         off += k
+
+
+def test_images_need_only_element_alignment(P):  # noqa: F811
+    net = P.WeightPredictor(R, seed=6)
+    img, cs = _inputs(3, seed=12)
+    I, Cs = torch.as_tensor(img, device="cuda"), torch.as_tensor(cs, device="cuda")
+    flat = torch.empty(I.numel() + 1, device="cuda")
+    shifted = flat[1:].view(I.shape)
+    shifted.copy_(I)
+    assert shifted.data_ptr() % 16 == 4
+    assert torch.equal(net.forward(shifted, Cs, tensor_cores=True), net.forward(I, Cs, tensor_cores=True))
