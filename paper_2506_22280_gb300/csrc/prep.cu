@@ -81,14 +81,23 @@ __global__ void __launch_bounds__(128) k_prep_ffd(GaussPtrs g, const __grid_cons
   }
 }
 
-// (2) One thread per (Gaussian, group of kPrepGroup projections): the deformation-informed warp (Eq. 7-8)
+// (2) One thread per (Gaussian, group of `group` projections): the deformation-informed warp (Eq. 7-8)
 // and the projection record of each projection of the group that renders the Gaussian's scan.
-// Record (b, n) of scan-local Gaussian n sits at b * nmax + n.  Grid: (ceil(n / 128), ceil(P / kPrepGroup)).
+// Record (b, n) of scan-local Gaussian n sits at b * nmax + n.  Grid: (ceil(n / 128), ceil(P / group)).  A group
+// shares the loads of the Gaussian and its FFD (12 R + 11 values); a thread's projections follow one another, so the
+// largest group that still fills the chip four times over (5 CTAs on each of 152 SMs) is taken.  Groups of 16 in every
+// call against this rule: 2,000 Gaussians, 16 projections 23 -> 6.4 us; 100k, 16 (782 CTAs, a second wave of 22) 56 -> 48;
+// 33k, 7 14.3 -> 12.7; 100k, 128 the same groups.
 constexpr int kPrepGroup = 16;
+int prep_group(int blocks, int P) {
+  int group = kPrepGroup;
+  while (group > 1 && (long long)blocks * ((P + group - 1) / group) < 4 * 5 * 152) group >>= 1;
+  return group;
+}
 template <int R>
 __global__ void __launch_bounds__(128, 5) k_prep_fwd(GaussPtrs g, const __grid_constant__ ScanTable sc,
                                                   const float* __restrict__ w, const __grid_constant__ ViewsParam views,
-                                                  int P, float c2, int tile, float4* __restrict__ rec,
+                                                  int P, int group, float c2, int tile, float4* __restrict__ rec,
                                                   uint32_t* __restrict__ counts, uint2* __restrict__ tbox,
                                                   uint8_t* __restrict__ bcost, const float* __restrict__ ffd,
                                                   int* status) {
@@ -107,8 +116,8 @@ __global__ void __launch_bounds__(128, 5) k_prep_fwd(GaussPtrs g, const __grid_c
   }
   const bool finite_in = isfinite(G.mu0[0] + G.mu0[1] + G.mu0[2] + G.s[0] + G.s[1] + G.s[2] + G.qnorm + G.rho);
   if (!finite_in && blockIdx.y == 0) set_status(status, DIGS_ERR_NONFINITE);
-  const int b1 = min(P, ((int)blockIdx.y + 1) * kPrepGroup);
-  for (int b = (int)blockIdx.y * kPrepGroup; b < b1; ++b) {
+  const int b1 = min(P, ((int)blockIdx.y + 1) * group);
+  for (int b = (int)blockIdx.y * group; b < b1; ++b) {
     const ViewC& v = views.v[b];
     if (v.scan != s) continue;
     const float* wb = w + (size_t)v.w_row * R;
@@ -160,10 +169,11 @@ cudaError_t launch_prep_fwd(const GaussPtrs& g, const ScanTable& sc, const Latti
     if (e != cudaSuccess) return e;
   }
   dim3 grid((g.n + 127) / 128);
-  dim3 grid2(grid.x, (P + kPrepGroup - 1) / kPrepGroup);
+  const int group = prep_group(grid.x, P);
+  dim3 grid2(grid.x, (P + group - 1) / group);
 #define DIGS_PREP(RR)                                                                                        \
   k_prep_ffd<RR><<<grid, 128, 0, st>>>(g, sc, L, phi, ws.ffd);                                                \
-  k_prep_fwd<RR><<<grid2, 128, 0, st>>>(g, sc, w, views, P, c2, ws.tile, ws.rec, ws.counts, ws.tbox, ws.bcost, \
+  k_prep_fwd<RR><<<grid2, 128, 0, st>>>(g, sc, w, views, P, group, c2, ws.tile, ws.rec, ws.counts, ws.tbox, ws.bcost, \
                                         ws.ffd, ws.status)
   switch (L.R) {
     case 1: DIGS_PREP(1); break;
