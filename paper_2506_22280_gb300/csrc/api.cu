@@ -284,8 +284,8 @@ digs_status bin(Call& c, const float* phi, const float* w) {
     DIGS_TRY(sort_pairs(ws.keys, ws.vals, ws.keys_alt, ws.vals_alt, ws.n_pairs, ws.cap, ws.offsets, ws.n, c.P,
                         ws.T, ws.n_sort_blocks, ws.seg, ws.hist, ws.scan_tmp, ws.ranges, &sk, &sv, c.st));
     ws.srid = sv;
+    DIGS_TRY(tile_order(ws.ranges, c.P * ws.T, ws.order, c.st));
   }
-  DIGS_TRY(tile_order(ws.ranges, c.P * ws.T, ws.order, c.st));
   mark(c, 3);
   return DIGS_OK;
 }

@@ -80,7 +80,7 @@ constexpr int kDirectMaxTiles = 1024;
 int bin_chunks(int n, int T);
 cudaError_t bin_direct(const Workspace& ws, cudaStream_t st);
 // order[P * T]: (projection, tile) indices by descending range length (power-of-two classes).
-cudaError_t tile_order(const uint2* ranges, int n, uint32_t* order, cudaStream_t st);
+cudaError_t tile_order(uint2* ranges, int n, uint32_t* order, cudaStream_t st);
 
 // prep.cu
 cudaError_t launch_ffd_eval(const LatticeC& L, const float* phi, const float* x, int n, float* U, float* dU,
