@@ -43,11 +43,11 @@ __device__ __forceinline__ void warp_reduce_scatter48(float v[48], int lane) {
 // d_j beta for the 64 nodes around x (Eq. 10 differentiated); lanes in the same lattice cell are summed
 // over the warp first.  GU / GdU: this thread's dL/du_r and
 // dL/d(grad u_r), read from shared memory at stride `st`.  Lanes with valid == false contribute nothing
-// but take part in the warp collectives.
+// but take part in the warp collectives.  [z0, z1): the z planes of nodes.
 template <int R>
 __device__ __forceinline__ void ffd_scatter_warp(float* __restrict__ g_phi_all, long long phi_stride, int scan,
                                                  const LatticeC& L, const float x[3], bool valid, const float* GU,
-                                                 const float* GdU, int st) {
+                                                 const float* GdU, int st, int z0, int z1) {
   const int lane = threadIdx.x & 31;
   int f[3];
   float u[3];
@@ -80,7 +80,7 @@ __device__ __forceinline__ void ffd_scatter_warp(float* __restrict__ g_phi_all, 
 #pragma unroll
     for (int c = 0; c < 9; ++c) gdu[c] = valid ? GdU[(r * 9 + c) * st] : 0.f;
 #pragma unroll 1
-    for (int n3 = 0; n3 < 4; ++n3) {
+    for (int n3 = z0; n3 < z1; ++n3) {
       const float bz = n3 == 0 ? B[2][0] : n3 == 1 ? B[2][1] : n3 == 2 ? B[2][2] : B[2][3];
       const float dbz = n3 == 0 ? dB[2][0] : n3 == 1 ? dB[2][1] : n3 == 2 ? dB[2][2] : dB[2][3];
       // v[(m * 4 + l) * 3 + c] = beta gu_c + sum_j gdu_cj d_j beta for node (l, m, n3); zero unless `on`
@@ -400,18 +400,22 @@ __global__ void __launch_bounds__(128) k_ffd_hessian(GaussPtrs g, const __grid_c
   for (int c = 0; c < 18; ++c) out[(size_t)(r * 18 + c) * g.n + n] = H[c];
 }
 
-// (2) Per Gaussian: from the summed pair adjoints, the FFD backward and the reference-parameter gradients.
-template <int R>
-__global__ void __launch_bounds__(32 * R, 4) k_gauss_bwd(
+// (2) Per Gaussian: from the summed pair adjoints, the FFD backward and the reference-parameter gradients.  Z warps share
+// a rank's 4 planes of nodes.  What bounds it: the chain of shuffles and atomics of a plane in small clouds, the
+// atomics of unordered ones.  Z = 4 where one warp per rank leaves the chip idle: up to kSplitWarps of them (16 an SM).
+// 2,000 Gaussians of two ranks 13.2 -> 8.4 us, 33k unordered ones 61 -> 57.
+constexpr int kSplitWarps = 16 * 152;
+template <int R, int Z>
+__global__ void __launch_bounds__(32 * R * Z, Z == 1 ? 4 : 1) k_gauss_bwd(
     GaussPtrs g, const __grid_constant__ ScanTable sc, LatticeC L, const float* __restrict__ ffd,
     const float* __restrict__ ffd2,
     const float* __restrict__ gsum, float* __restrict__ dens_grad, float* __restrict__ g_mu0,
     float* __restrict__ g_scale, float* __restrict__ g_quat, float* __restrict__ g_rho, float* __restrict__ g_phi) {
-  // warp r takes rank r of the CTA's 32 Gaussians: dL/du_r (3) then dL/d(grad u_r) (9), lane-fastest
-  __shared__ float Gs[R][12 * 32];
+  // warp z R + r takes rank r (and planes z) of the CTA's 32 Gaussians: dL/du_r (3) then dL/d(grad u_r) (9), lane-fastest
+  __shared__ float Gs[R * Z][12 * 32];
   __shared__ float gpart[R][3][32];  // each rank's share of dL/dmu0
   const int N = g.n;
-  const int lane = threadIdx.x & 31, r = (int)(threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, rz = (int)(threadIdx.x >> 5), r = rz % R, z = rz / R;
   const int n = blockIdx.x * 32 + lane;
   const bool valid = n < N;
   const int scan = valid ? scan_of(sc, n) : 0;
@@ -429,6 +433,7 @@ __global__ void __launch_bounds__(32 * R, 4) k_gauss_bwd(
     // u_r and grad u_r are evaluated at mu0: dL/dmu0 += (grad u_r)^T dL/du_r + H_r : dL/d(grad u_r)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
+      if (z != 0) break;  // one warp of the rank's
       const float* du = ffd + (size_t)(3 * R + r * 9 + c * 3) * N + n;   // d u_rc / dx_m, m = 0..2
       const float* h = ffd2 + (size_t)(r * 18 + c * 6) * N + n;          // xx, yy, zz, xy, xz, yz
       const float hxx = h[0], hyy = h[(size_t)N], hzz = h[(size_t)2 * N];
@@ -441,17 +446,17 @@ __global__ void __launch_bounds__(32 * R, 4) k_gauss_bwd(
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    Gs[r][c * 32 + lane] = GU[c];
-    gpart[r][c][lane] = gm[c];
+    Gs[rz][c * 32 + lane] = GU[c];
+    if (z == 0) gpart[r][c][lane] = gm[c];
   }
 #pragma unroll
-  for (int c = 0; c < 9; ++c) Gs[r][(3 + c) * 32 + lane] = GdU[c];
-  // each lane reads back only its own column of Gs[r], so no barrier is needed before the scatter
+  for (int c = 0; c < 9; ++c) Gs[rz][(3 + c) * 32 + lane] = GdU[c];
+  // each lane reads back only its own column of Gs[rz], so no barrier is needed before the scatter
   const size_t rank_stride = (size_t)L.nx * L.ny * L.nz * 3;
-  ffd_scatter_warp<1>(g_phi + r * rank_stride, sc.phi_stride, scan, L, mu0, valid, &Gs[r][lane], &Gs[r][3 * 32 + lane],
-                      32);
+  ffd_scatter_warp<1>(g_phi + r * rank_stride, sc.phi_stride, scan, L, mu0, valid, &Gs[rz][lane], &Gs[rz][3 * 32 + lane],
+                      32, z * (4 / Z), (z + 1) * (4 / Z));
   __syncthreads();
-  if (r != 0 || !valid) return;
+  if (rz != 0 || !valid) return;
   const float* q = gsum + n;
   float gmu0[3], gs[3], gth[3];
 #pragma unroll
@@ -485,6 +490,7 @@ cudaError_t launch_chain_bwd(const GaussPtrs& g, const ScanTable& sc, const Latt
                              cudaStream_t st) {
   if (g.n <= 0) return cudaSuccess;
   dim3 gb(chain_blocks(g.n)), gp(pair_sum_blocks(g.n));
+  const int gauss_ctas = (g.n + 31) / 32;
 #define DIGS_CH(RR)                                                                                             \
   {                                                                                                             \
     static bool configured = false;                                                                             \
@@ -496,9 +502,12 @@ cudaError_t launch_chain_bwd(const GaussPtrs& g, const ScanTable& sc, const Latt
   k_ffd_hessian<<<dim3(gb.x, RR), 128, 0, st>>>(g, sc, L, phi, ws.ffd2);                                      \
   k_pair_sum<RR><<<gp, kSlots * 32, pair_sum_smem<RR>(), st>>>(g, sc, ws.ffd, w, views, P, ws.counts, ws.grec,   \
                                                               ws.gsum, ws.gw_part);                            \
-  k_gauss_bwd<RR><<<(g.n + 31) / 32, 32 * RR, 0, st>>>(g, sc, L, ws.ffd, ws.ffd2, ws.gsum, dens_grad, g_mu0,     \
-                                                       g_scale,                                              \
-                                               g_quat, g_rho, g_phi)
+  if ((long long)gauss_ctas * RR <= kSplitWarps)                                                               \
+    k_gauss_bwd<RR, 4><<<gauss_ctas, 32 * RR * 4, 0, st>>>(g, sc, L, ws.ffd, ws.ffd2, ws.gsum, dens_grad, g_mu0, \
+                                                           g_scale, g_quat, g_rho, g_phi);                     \
+  else                                                                                                         \
+    k_gauss_bwd<RR, 1><<<gauss_ctas, 32 * RR, 0, st>>>(g, sc, L, ws.ffd, ws.ffd2, ws.gsum, dens_grad, g_mu0,   \
+                                                       g_scale, g_quat, g_rho, g_phi)
   switch (L.R) {
     case 1: DIGS_CH(1); break;
     case 2: DIGS_CH(2); break;
