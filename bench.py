@@ -593,7 +593,7 @@ def cnn_measurement(pkg, device, B=256, R=3, reps=20):
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     peak = float(peaks.get("bf16_tflops", 1900.0))
     out["train_step_speedup"] = out["train_step_ms_fp32_simt"] / out["train_step_ms_tensor_cores"]
-    out["roofline"] = {"bound": "tensor", "kernel": "k_gemm_tc (whole training step)", "achieved": achieved,
+    out["roofline"] = {"bound": "tensor", "kernel": "k_conv, k_conv_dw, k_cnn_gemm (whole training step)", "achieved": achieved,
                        "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                        "peak_basis": "measured dense BF16 burst" if "bf16_tflops" in peaks else "fallback 1.9 PFLOP/s",
                        "flops_per_step": flops}

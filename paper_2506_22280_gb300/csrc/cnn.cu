@@ -12,7 +12,7 @@
 //   data grad    dX[M][K] = dY[M][N] W[N][K]
 //   weight grad  dW[N][K] = dY[M][N]^T X[M][K]     (split over M, partials summed in a fixed order)
 // The forward and backward run either in FP32 on the SIMT pipes or, with DIGS_CNN_TENSOR_CORES, with the
-// large GEMMs (the convolutions and the 8194-wide layer) on the tensor cores: BF16 operands rounded from
+// large GEMMs (the convolutions but the first, and the 8194-wide layer) on the tensor cores: BF16 operands rounded from
 // the FP32 activations, gradients and weights, FP32 accumulation; the R-wide output layer stays FP32.
 // Inference reads BF16 weights and activations and runs its large GEMMs on the tensor cores.
 #include <cuda_bf16.h>
@@ -248,8 +248,8 @@ CnnNet cnn_net(const NetPtrs<float>& N) {
 }
 
 // Forward keeping every activation in the workspace for the backward.  tc: the tensor-core path of
-// cnn_tc.cu up to the dense layer's output (BF16 activations), else FP32 SIMT GEMMs over im2col
-// matrices; the R-wide output layer is FP32 either way.
+// cnn_tc.cu up to the dense layer's output (BF16 activations), else the FP32 SIMT GEMMs of cnn_f32.cu; the
+// R-wide output layer is FP32 either way.
 cudaError_t forward_f32(const NetPtrs<float>& N, int R, const float* img, const float* cs, int B, const CnnWs& w,
                         bool tc, cudaStream_t st) {
   if (tc) {

@@ -1,6 +1,6 @@
 // Dense GEMM on the fifth-generation tensor cores (tcgen05, sm_103a): C = op(A) op(B) with BF16 operands
 // and FP32 accumulation in tensor memory, behind digs_gemm_bf16 (FP32 operands rounded while staged).
-// The CNN's own layers run on the kernels of cnn_tc.cu, which read BF16 activations in place.
+// The CNN's own layers run on the kernels of cnn_conv.cu and cnn_tc.cu, which read BF16 activations in place.
 //
 // C(m, n) = sum_k A(m, k) B(k, n); A(m, k) = AT ? A[k lda + m] : A[m lda + k] and
 // B(k, n) = BT ? B[n ldb + k] : B[k ldb + n], FP32 in global memory.  One CTA of 128 threads per
