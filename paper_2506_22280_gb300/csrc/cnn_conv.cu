@@ -24,10 +24,8 @@
 // each, on the threads that also ran the epilogue, and stored 16 bytes per lane at a distance of 128.
 // Launch times at batch 256, layers 1 / 2 / 3, before and now: forward 97 / 62 / 39 -> 32 / 19 / 12 us, data
 // gradient 167 / 102 / 51 -> 33 / 28 / 18, weight gradient 103 / 67 / 35 -> 23 / 17 / 13; the training step
-// as a whole 978 -> 443 us, inference of 680 projections 745 -> 378 us.  The multiply-adds of every output element are added in
+// 978 -> 443 us, inference of 680 projections 745 -> 378 us.  The multiply-adds of every output element are added in
 // the same order as before.
-// Layer 1's weights (48 and 36 KB) stay in shared memory (training step 411 -> 406 us), the others' come with each
-// slice.
 // One warp issues the copies, one the MMAs, four run the epilogue on the other half of the tensor memory; CTAs are
 // persistent, one per SM.  Every wait is bounded: a role that gives up sets *status, waits for what it has in
 // flight and leaves; the sums that follow turn into NaN (k_sum_z).
@@ -138,27 +136,23 @@ template <int L>
 struct Fwd {
   using G = Geo<L>;
   static constexpr bool kMask = false;
-  static constexpr int kCols = G::N, kSlices = G::C == 32 ? 6 : 9 * G::C / 64, kStages = L == 1 ? 8 : 5;
+  static constexpr int kCols = G::N, kSlices = G::C == 32 ? 6 : 9 * G::C / 64, kStages = L == 1 ? 6 : 5;
   static constexpr int kBBytes = G::N * 128, kIoBoxes = G::N / 64, kIo = 1, kSums = 1;
-  static constexpr int kResident = L == 1 ? kSlices * kBBytes : 0;
-  static __device__ uint32_t b_bytes(int) { return kBBytes; }
-  static __device__ uint32_t b_off(int s) { return s * kBBytes; }
-  static __device__ void load_b(const CUtensorMap* mb, uint64_t* bar, uint32_t sb, int s, int) {
-    int k = s * 64;
-    if constexpr (G::C == 32) k = (s >> 1) * 96 + (s & 1) * 32;
-    load2(sb, mb, bar, k, 0);
-  }
-  static __device__ void load_a(const CUtensorMap* ma, uint64_t* bar, uint32_t sa, int s, int t) {
-    int c0, dx, py, dy;
+  static __device__ uint32_t slice_bytes(int) { return kSlice + kBBytes; }
+  static __device__ void load(const CUtensorMap* ma, const CUtensorMap* mb, uint64_t* bar, uint32_t sa, uint32_t sb,
+                              int s, int t, int) {
+    int c0, dx, py, dy, k;
     if constexpr (G::C == 32) {
       const int ky = s >> 1, pair = s & 1;
-      c0 = 0; dx = pair - 1; py = ky != 1; dy = ky == 0 ? -1 : 0;
+      c0 = 0; dx = pair - 1; py = ky != 1; dy = ky == 0 ? -1 : 0; k = ky * 96 + pair * 32;
     } else {
       constexpr int Hf = G::C / 64;
       const int tap = s / Hf, half = s % Hf, ky = tap / 3, kx = tap % 3;
       c0 = (kx != 1 ? G::C : 0) + half * 64; dx = kx == 0 ? -1 : 0; py = ky != 1; dy = ky == 0 ? -1 : 0;
+      k = tap * G::C + half * 64;
     }
     load5(sa, ma, bar, c0, dx, py, G::row(t) + dy, G::img(t));
+    load2(sb, mb, bar, k, 0);
   }
   static __device__ void mma(uint32_t tmem, uint32_t sa, uint32_t sb, int s) {
     constexpr uint32_t idesc = tc::idesc_bf16(128, G::N, false, false);
@@ -198,19 +192,15 @@ struct Dx {
   using G = Geo<L>;
   static constexpr bool kMask = true;
   static constexpr int CC = G::C < 64 ? G::C : 64, Hf = G::N / 64;
-  static constexpr int kCols = 4 * CC, kSlices = 4 * Hf, kStages = CC == 32 ? 6 : 3;
+  static constexpr int kCols = 4 * CC, kSlices = 4 * Hf, kStages = CC == 32 ? 4 : 3;
   static constexpr int kBBytes = 4 * CC * 128, kIoBoxes = 4 * CC / 64, kIo = CC == 32 ? 2 : 1, kSums = CC;
   static __device__ int blocks(int shift) { return shift == 0 ? 4 : (shift == 3 ? 1 : 2); }
   static __device__ int shift_of(int s) { return 3 - s / Hf; }  // 2 dy + dx, (1, 1) first
-  static constexpr int kResident = L == 1 ? 9 * CC * 128 : 0;
-  static __device__ uint32_t b_bytes(int s) { return blocks(shift_of(s)) * CC * 128; }
-  static __device__ uint32_t b_off(int s) { return (s == 0 ? 0 : 2 * s - 1) * CC * 128; }  // resident: blocks 1, 2, 2, 4
-  static __device__ void load_a(const CUtensorMap* ma, uint64_t* bar, uint32_t sa, int s, int t) {
-    const int shift = shift_of(s);
-    load4(sa, ma, bar, s % Hf * 64, shift & 1, G::row(t) + (shift >> 1), G::img(t));
-  }
-  static __device__ void load_b(const CUtensorMap* mb, uint64_t* bar, uint32_t sb, int s, int chunk) {
+  static __device__ uint32_t slice_bytes(int s) { return kSlice + blocks(shift_of(s)) * CC * 128; }
+  static __device__ void load(const CUtensorMap* ma, const CUtensorMap* mb, uint64_t* bar, uint32_t sa, uint32_t sb,
+                              int s, int t, int chunk) {
     const int shift = shift_of(s), half = s % Hf, nb = blocks(shift);
+    load4(sa, ma, bar, half * 64, shift & 1, G::row(t) + (shift >> 1), G::img(t));
     const int base = (shift == 0 ? 0 : 2 + 2 * shift) * Hf + half * nb + chunk * 9 * Hf;
     for (int i = 0; i < nb; ++i) load2(sb + i * CC * 128, mb, bar, 0, (base + i) * CC);
   }
@@ -285,9 +275,10 @@ struct Dx {
 
 template <class P>
 struct Smem {
-  static constexpr int kStage = kSlice + (P::kResident ? 0 : P::kBBytes);
+  static constexpr int kStage = kSlice + P::kBBytes;
   static constexpr int kIoBytes = P::kIoBoxes * kSlice;
-  static constexpr size_t kBytes = 1024 + P::kStages * kStage + P::kResident + P::kIo * kIoBytes + 256 + 512;  // barriers, bias
+  static constexpr int kBars = 1024 + P::kStages * kStage + P::kIo * kIoBytes;  // from the aligned base: - 1024
+  static constexpr size_t kBytes = kBars + 256 + 512;                          // barriers, bias
 };
 
 // Tiles blockIdx.x, blockIdx.x + gridDim.x, ... of 128 rows.  Double-buffered accumulator (2 kCols columns).
@@ -300,11 +291,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int kSt = P::kStages;
   extern __shared__ unsigned char smem_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* io = sm + kSt * S::kStage + P::kResident;
+  uint8_t* io = sm + kSt * S::kStage;
   uint64_t* full = (uint64_t*)(io + P::kIo * S::kIoBytes);
   uint64_t *empty = full + kSt, *tfull = empty + kSt, *tempty = tfull + 2, *iofull = tempty + 2, *ioempty = iofull + 2,
-           *drain = ioempty + 2, *bfull = drain + 1;
-  uint32_t* slot = (uint32_t*)(bfull + 1);
+           *drain = ioempty + 2;
+  uint32_t* slot = (uint32_t*)(drain + 1);
   float* sbias = (float*)((uint8_t*)full + 256);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, chunk = blockIdx.y;
   if (threadIdx.x == 0) {
@@ -319,7 +310,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(ioempty + s, 1);
     }
     tc::mbar_init(drain, 1);
-    tc::mbar_init(bfull, 1);
     tc::mbar_init_fence();
   }
   if (!P::kMask && threadIdx.x < P::kCols) sbias[threadIdx.x] = bias[threadIdx.x];
@@ -328,23 +318,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *slot, sbase = tc::smem_u32(sm), iobase = tc::smem_u32(io);
-  const uint32_t bbase = sbase + kSt * S::kStage;  // the weights, where all of them fit
   bool ok = true;
   if (warp == 0) {
     if (lane == 0) {
       unsigned g = 0, i = 0;  // slices and activation tiles issued
-      if (P::kResident) {
-        expect_tx(bfull, P::kResident);
-        for (int s = 0; s < P::kSlices; ++s) P::load_b(&mb, bfull, bbase + P::b_off(s), s, chunk);
-      }
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         for (int s = 0; s < P::kSlices; ++s, ++g) {
           const unsigned st = g % kSt;
           if (g >= kSt && !(ok = tc::mbar_wait(empty + st, (g / kSt - 1) & 1u, limit))) break;
-          expect_tx(full + st, kSlice + (P::kResident ? 0 : P::b_bytes(s)));
+          expect_tx(full + st, P::slice_bytes(s));
           const uint32_t sa = sbase + st * S::kStage;
-          P::load_a(&ma, full + st, sa, s, t);
-          if (!P::kResident) P::load_b(&mb, full + st, sa + kSlice, s, chunk);
+          P::load(&ma, &mb, full + st, sa, sa + kSlice, s, t, chunk);
         }
         if (P::kMask && ok) {  // the activations of the tile, once its buffer has been stored from
           const unsigned b = i % P::kIo;
@@ -354,7 +338,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       // every copy has landed before the CTA may leave
-      if (P::kResident) tc::mbar_wait(bfull, 0, tc::kWaitLimit);
       for (unsigned k = g > kSt ? g - kSt : 0; k < g; ++k) tc::mbar_wait(full + k % kSt, (k / kSt) & 1u, tc::kWaitLimit);
       for (unsigned k = i > P::kIo ? i - P::kIo : 0; k < i; ++k)
         tc::mbar_wait(iofull + k % P::kIo, (k / P::kIo) & 1u, tc::kWaitLimit);
@@ -362,7 +345,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       unsigned g = 0, i = 0;
-      if (P::kResident) ok = tc::mbar_wait(bfull, 0, limit);
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++i) {
         if (i >= 2 && !(ok = tc::mbar_wait(tempty + (i & 1), (i / 2 - 1) & 1u, limit))) break;
         tc::fence_after();
@@ -371,7 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!(ok = tc::mbar_wait(full + st, (g / kSt) & 1u, limit))) break;
           tc::fence_after();
           const uint32_t sa = sbase + st * S::kStage;
-          P::mma(tmem + (i & 1) * P::kCols, sa, P::kResident ? bbase + P::b_off(s) : sa + kSlice, s);
+          P::mma(tmem + (i & 1) * P::kCols, sa, sa + kSlice, s);
           tc::mma_commit(empty + st);
         }
         if (ok) tc::mma_commit(tfull + (i & 1));
