@@ -19,7 +19,9 @@
 // Weight gradient: dW[(tap, ci)][co], K = pixels; a CTA holds three 128-row tiles of (tap, ci) and reads dY once
 // for them, its share of the pixels one 64-pixel box after another.
 //
-// What bounds them: the fill of shared memory from L2 and HBM (the MMAs take less than a third of the time).
+// What bounds them: the latency of a tile's chain of copies, MMAs and epilogue with one tile after another on an SM; at
+// batch 256 HBM runs at 15 to 36 % of its peak, the L2 at 15 to 22 % and the tensor pipe at 14 to 30 %.  (Keeping
+// layer 1's weights in shared memory, a third of its fill, changed nothing: 411 and 406 us a training step.)
 // The form before this one gathered 16 bytes per thread and cp.async, with the address arithmetic of a tap for
 // each, on the threads that also ran the epilogue, and stored 16 bytes per lane at a distance of 128.
 // Launch times at batch 256, layers 1 / 2 / 3, before and now: forward 97 / 62 / 39 -> 32 / 19 / 12 us, data
@@ -27,7 +29,7 @@
 // 978 -> 443 us, inference of 680 projections 745 -> 378 us.  The multiply-adds of every output element are added in
 // the same order as before.
 // One warp issues the copies, one the MMAs, four run the epilogue on the other half of the tensor memory; CTAs are
-// persistent, one per SM.  Every wait is bounded: a role that gives up sets *status, waits for what it has in
+// persistent, one per SM (layer 1's forward two: 411 -> 401 us a training step, 353 -> 343 the inference).  Every wait is bounded: a role that gives up sets *status, waits for what it has in
 // flight and leaves; the sums that follow turn into NaN (k_sum_z).
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -136,7 +138,7 @@ template <int L>
 struct Fwd {
   using G = Geo<L>;
   static constexpr bool kMask = false;
-  static constexpr int kCols = G::N, kSlices = G::C == 32 ? 6 : 9 * G::C / 64, kStages = L == 1 ? 6 : 5;
+  static constexpr int kCols = G::N, kSlices = G::C == 32 ? 6 : 9 * G::C / 64, kStages = L == 1 ? 3 : 5, kCtas = L == 1 ? 2 : 1;
   static constexpr int kBBytes = G::N * 128, kIoBoxes = G::N / 64, kIo = 1, kSums = 1;
   static __device__ uint32_t slice_bytes(int) { return kSlice + kBBytes; }
   static __device__ void load(const CUtensorMap* ma, const CUtensorMap* mb, uint64_t* bar, uint32_t sa, uint32_t sb,
@@ -192,7 +194,7 @@ struct Dx {
   using G = Geo<L>;
   static constexpr bool kMask = true;
   static constexpr int CC = G::C < 64 ? G::C : 64, Hf = G::N / 64;
-  static constexpr int kCols = 4 * CC, kSlices = 4 * Hf, kStages = CC == 32 ? 4 : 3;
+  static constexpr int kCols = 4 * CC, kSlices = 4 * Hf, kStages = CC == 32 ? 4 : 3, kCtas = 1;
   static constexpr int kBBytes = 4 * CC * 128, kIoBoxes = 4 * CC / 64, kIo = CC == 32 ? 2 : 1, kSums = CC;
   static __device__ int blocks(int shift) { return shift == 0 ? 4 : (shift == 3 ? 1 : 2); }
   static __device__ int shift_of(int s) { return 3 - s / Hf; }  // 2 dy + dx, (1, 1) first
@@ -283,7 +285,7 @@ struct Smem {
 
 // Tiles blockIdx.x, blockIdx.x + gridDim.x, ... of 128 rows.  Double-buffered accumulator (2 kCols columns).
 template <class P>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, P::kCtas)
     k_conv(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, const __grid_constant__ CUtensorMap mio,
            const __grid_constant__ CUtensorMap mout, const float* __restrict__ bias, float* __restrict__ colpart, int colpitch,
            int n_tiles, unsigned* status, unsigned limit) {
@@ -597,7 +599,7 @@ cudaError_t forward(const uint16_t* act, const uint16_t* w, const float* bias, i
       !encode(&o, out, 3, Dims{{G::N, px, (cuuint64_t)B}, {1, G::N, (cuuint64_t)pitch}, {64, 128 / G::kImgs, G::kImgs}}))
     return cudaErrorInvalidValue;
   const int tiles = G::tiles(B);
-  return launch<Fwd<L>>(a, b, o, o, bias, nullptr, tiles, std::min(tiles, kSms), 1, status, st);
+  return launch<Fwd<L>>(a, b, o, o, bias, nullptr, tiles, std::min(tiles, Fwd<L>::kCtas * kSms), 1, status, st);
 }
 
 template <int L>
