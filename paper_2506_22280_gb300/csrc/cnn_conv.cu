@@ -656,8 +656,10 @@ cudaError_t cnn_conv_dx(int l, const uint16_t* dy, const uint16_t* wt, const uin
 
 int cnn_conv_dw_splits(int l, int B, long long part_floats) {
   const long long slices = (long long)B * kSide[l + 1] * kSide[l + 1] / 64;
-  const int groups = l == 1 ? Dw<1>::kGroups : (l == 2 ? Dw<2>::kGroups : Dw<3>::kGroups);
-  long long z = kSms / groups;
+  // 304 (tile of 128 rows, split) pairs, at least four boxes per split.  The line is that of the gathering kernels
+  // before: the same splits give the same sums, bit for bit, and so the same rounded weights after a step.
+  const int tiles = (9 * kChan[l] + 127) / 128;
+  long long z = (2 * kSms + tiles - 1) / tiles;
   z = std::min(z, std::max(1LL, slices / 4));
   z = std::min(z, std::max(1LL, part_floats / (9LL * kChan[l] * kChan[l + 1])));
   const long long per = (slices + z - 1) / z;
