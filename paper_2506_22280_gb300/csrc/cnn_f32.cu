@@ -347,6 +347,12 @@ int splits_for(int tiles, long long K, int least, long long n, long long room) {
 }
 int chunk_of(long long K, int z) { return (int)(((K + z - 1) / z + kBK - 1) / kBK * kBK); }
 
+// Gradients of the convolutions' outputs pass through two buffers in turn: layers 0 and 2 in dy[0], 1 and 3 in dy[1]
+// (floats per image).
+constexpr int out_floats(int l) { return kEdge[l + 1] * kEdge[l + 1] * kCh[l + 1]; }
+constexpr int kDyFloats[2] = {out_floats(0), out_floats(1)};
+static_assert(out_floats(2) <= kDyFloats[0] && out_floats(3) <= kDyFloats[1], "every layer's gradient fits its buffer");
+
 struct Layer {
   int H, lwo, lc, ln, rows, N, K, C;
 };
@@ -377,8 +383,7 @@ size_t cnn_f32_layout(void* base, int B, CnnF32* t) {
   w.img = take((size_t)B * 128 * 128);
   for (int l = 0; l < 3; ++l) w.act[l] = take((size_t)B * kEdge[l + 1] * kEdge[l + 1] * kCh[l + 1]);
   w.feat = take((size_t)B * kFeatIn);
-  w.dy[0] = take((size_t)B * 4096 * 32);
-  w.dy[1] = take((size_t)B * 1024 * 64);
+  for (int k = 0; k < 2; ++k) w.dy[k] = take((size_t)B * kDyFloats[k]);
   w.part_floats = std::max<long long>(16LL * B * kHid, 6LL << 20);
   w.part = take((size_t)w.part_floats);
   if (t) *t = w;
@@ -413,7 +418,7 @@ cudaError_t cnn_f32_backward(const CnnNet& net, int B, const CnnF32& t, const Cn
   // dense layer: dW1[n][f] = sum_b dh[b][n] feat[b][f]; dY of the last convolution
   F32_TRY((gemm<64, 64>(PlainR{dh, kHid, kHid, B}, PlainR{t.feat, kFeatIn, kFeatIn, B}, EpiPart{g.w1, 0, kHid, kFeatIn}, kHid,
                         kFeatIn, B, 1, B, 0, st)));
-  float* dy = t.dy[0];
+  float* dy = t.dy[1];
   F32_TRY((gemm<64, 64>(PlainK{dh, kHid, B, kHid}, PlainR{net.w1, kFeatIn, kFeat, kHid}, EpiDfeat{dy, t.feat, B}, B, kFeat, kHid,
                         1, kHid, 0, st)));
   for (int l = 3; l >= 1; --l) {
@@ -425,7 +430,7 @@ cudaError_t cnn_f32_backward(const CnnNet& net, int B, const CnnF32& t, const Cn
     F32_TRY((gemm<64, 64>(DyR{dy, a.N, a.rows}, X, EpiPart{t.part, (long long)a.N * a.K, a.N, a.K}, a.N, a.K, a.rows, Z,
                           chunk_of(a.rows, Z), 0, st)));
     F32_TRY(cnn_sum_splits(t.part, Z, (long long)a.N * a.K, nullptr, 1, g.w[l], st));
-    float* dx = dy == t.dy[0] ? t.dy[1] : t.dy[0];
+    float* dx = t.dy[(l - 1) & 1];
     const ParityK A{dy, a.lwo, a.ln, a.rows};
     const ClassWR W{net.w[l], a.ln, a.C, on16(net.w[l])};
     const EpiDx ep{dx, t.act[l - 1], a.lwo, a.rows, a.C};
