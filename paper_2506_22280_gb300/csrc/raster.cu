@@ -552,8 +552,9 @@ __global__ void __launch_bounds__(32 * W, 28 / W) k_raster_bwd(const float4* __r
   const int i0 = max(0, (dead - r0) / kPer);  // the first round with a live record
   auto fetch = [&](int i) {  // one commit group per call and thread, empty or not
     if (i < WR) {
-      const int n = n0 + __shfl_sync(0xffffffffu, of_rank, r0 + i * kPer + half);
-      if (hl < DIGS_REC_F4) cp_async16(&sbuf[warp][i & 1][half][hl], rec + (unsigned)n * DIGS_REC_F4 + hl);
+      const int rank = r0 + i * kPer + half, n = n0 + __shfl_sync(0xffffffffu, of_rank, rank);
+      // not for a dead rank: its lane may lie past the projection's records
+      if (rank >= dead && hl < DIGS_REC_F4) cp_async16(&sbuf[warp][i & 1][half][hl], rec + (unsigned)n * DIGS_REC_F4 + hl);
     }
     cp_async_commit();
   };
