@@ -149,39 +149,24 @@ struct FwdCfg {
   static constexpr int min_ctas = (NB == 1 ? 32 : 28) / warps;
 };
 
-// A record's share of the entries that the pixel loops read, the same for every block: with k = -log2(e) / 2 and
-// sg = |amp| (1 when |amp| lies outside [2^-40, 2^40]), the quadratic form times k / sg^2, t's slopes over sg,
-// kappa / k and amp / sg.  The loop then forms the exp2 argument k E = k num / D directly; num and t scaled by
-// 1 / sg^2 and 1 / sg scale D by 1 / sg^2 and leave E unchanged, so the SFU's rsqrt of the scaled D is
-// sg D^-1/2 (amp / sg, i.e. the sign of amp, multiplies both pixels of a lane at once).
-struct FwdScaled {
-  float n00, n01, n11, t1, t2, s1, kap, sgn;
+// A record as the pixel loops read it: with k = -log2(e) / 2 and sg = |amp| (1 when |amp| lies outside
+// [2^-40, 2^40]),
+//   (k n00 / sg^2, k n01x2 / sg^2, k n11 / sg^2, wn0 / sg), (wn1 / sg, kappa / k, amp / sg, -xc), (-yc, 1 / sg, 0, 0).
+// The loop then forms the exp2 argument k E = k num / D directly; num and t scaled by 1 / sg^2 and 1 / sg scale D by
+// 1 / sg^2 and leave E unchanged, so the SFU's rsqrt of the scaled D is sg D^-1/2 (amp / sg, i.e. the sign of amp,
+// multiplies both pixels of a lane at once).
+struct FwdEntry {
+  float4 q[3];
 };
-__device__ __forceinline__ FwdScaled scale_record(const float4& a, const float4& b, const float4& c) {
+__device__ __forceinline__ FwdEntry scale_record(const float4& a, const float4& b, const float4& c) {
   const float mag = fabsf(c.x);
   const bool fold = mag >= 0x1p-40f && mag <= 0x1p40f;
-  FwdScaled r;
-  r.s1 = fold ? __frcp_rn(mag) : 1.f;
-  r.sgn = fold ? copysignf(1.f, c.x) : c.x;
-  const float s2 = r.s1 * r.s1 * kNegHalfLog2e;
-  r.n00 = a.z * s2;
-  r.n01 = a.w * s2;
-  r.n11 = b.x * s2;
-  r.t1 = b.y * r.s1;
-  r.t2 = b.z * r.s1;
-  r.kap = b.w * (1.f / kNegHalfLog2e);
-  return r;
-}
-
-// The entry of one 8 x 8 block.  With (X, Y) the block centre's offset from the projected mean and (x, y) a
-// pixel's offset from the block centre (x, y in -3.5 ... 3.5),
-//   k num / sg^2 = a0 + x (a1 + x a2) + y (b0 + x b1 + y c),  t / sg = t0 + x t1 + y t2,
-// so that x and y are constants of the lane: a column costs four FMAs and a row three, with no offset to form.
-__device__ __forceinline__ void write_entry(const FwdScaled& r, float X, float Y, float4* ent) {
-  const float h0 = r.n00 * X, h1 = r.n11 * Y;
-  ent[0] = make_float4(r.n00, r.n01, fmaf(r.n01, Y, 2.f * h0), fmaf(r.n01, X, 2.f * h1));  // a2, b1, a1, b0
-  ent[1] = make_float4(fmaf(X, fmaf(r.n01, Y, h0), h1 * Y), fmaf(r.t1, X, fmaf(r.t2, Y, r.s1)), r.t1, r.n11);  // a0, t0, t1, c
-  ent[2] = make_float4(r.t2, r.kap, r.sgn, 0.f);
+  const float s1 = fold ? __frcp_rn(mag) : 1.f, s2 = s1 * s1;
+  FwdEntry e;
+  e.q[0] = make_float4(kNegHalfLog2e * a.z * s2, kNegHalfLog2e * a.w * s2, kNegHalfLog2e * b.x * s2, b.y * s1);
+  e.q[1] = make_float4(b.z * s1, b.w * (1.f / kNegHalfLog2e), fold ? copysignf(1.f, c.x) : c.x, -a.x);
+  e.q[2] = make_float4(-a.y, s1, 0.f, 0.f);
+  return e;
 }
 
 // Whether the 8 x 8 pixel block whose centre lies at (X, Y) from the projected mean can hold a pixel with
@@ -202,25 +187,29 @@ __device__ __forceinline__ bool ellipse_meets(float n00, float n01x2, float n11,
   return !(fminf(qx, qy) > lim);
 }
 
-// One entry at the lane's two pixels, x and YY = (y, y + 4) from the block centre: their exp2 arguments k E (a
-// pair counts where k E >= c2 k), and V / |X - s| as r 2^(k E).
+// One entry at the lane's two pixels, x and YY = (y, y + 4): their exp2 arguments k E (a pair counts where
+// k E >= c2 k), and V / |X - s| as r 2^(k E).  The form is evaluated about the mean, whose offset is formed first:
+// expanded about a block's centre instead it costs two operations fewer per entry, but its terms cancel near the mean
+// of a small Gaussian (root mean square error of E in FP32, about the mean and about the block's centre: 1e-7 and
+// 2.2e-7 at a sigma of 2.8 pixels, 6e-7 at 1, 6e-6 at 0.3, 5e-5 at 0.1).
 struct FwdPair {
   float ra, rb, ea, eb;
 };
 __device__ __forceinline__ FwdPair fwd_pair(const float4* en, float x, f2 YY) {
   const float4 q0 = en[0], q1 = en[1], q2 = en[2];
   // the lane's two pixels share their column: its terms are formed once
-  const f2 P = f2_fma(f2_dup(x), f2_pack(q0.x, q0.y), f2_pack(q0.z, q0.w));  // x a2 + a1, b0 + x b1
+  const float dx = x + q1.w;
   float p, bq;
-  f2_unpack(P, p, bq);
-  const float aq = fmaf(x, p, q1.x), tq = fmaf(x, q1.z, q1.y);
-  const f2 NUM = f2_fma(YY, f2_fma(f2_dup(q1.w), YY, f2_dup(bq)), f2_dup(aq));  // k num / sg^2
-  const f2 T = f2_fma(f2_dup(q2.x), YY, f2_dup(tq));                             // t / sg
-  const f2 D = f2_fma(T, T, f2_mul(f2_dup(q2.y), NUM));                          // D / sg^2
+  f2_unpack(f2_mul(f2_pack(q0.x, q0.y), f2_dup(dx)), p, bq);
+  const float aq = p * dx, tq = fmaf(q0.w, dx, q2.y);
+  const f2 DY = f2_add(YY, f2_dup(q2.x));
+  const f2 NUM = f2_fma(DY, f2_fma(f2_dup(q0.z), DY, f2_dup(bq)), f2_dup(aq));  // k num / sg^2
+  const f2 T = f2_fma(f2_dup(q1.x), DY, f2_dup(tq));                             // t / sg
+  const f2 D = f2_fma(T, T, f2_mul(f2_dup(q1.y), NUM));                          // D / sg^2
   const f2 RS = f2_rsqrt(D);                                                     // sg D^-1/2
   const f2 ARG = f2_mul(NUM, f2_mul(RS, RS));                                    // k E
   FwdPair r;
-  f2_unpack(f2_mul(RS, f2_dup(q2.z)), r.ra, r.rb);
+  f2_unpack(f2_mul(RS, f2_dup(q1.z)), r.ra, r.rb);
   f2_unpack(ARG, r.ea, r.eb);
   return r;
 }
@@ -247,8 +236,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
   const int gx = (tile % tiles_x) * TS + (sub & 1) * 16 + (NB == 1 ? (group & 1) * 8 : 0);
   const int gy = (tile / tiles_x) * TS + (sub >> 1) * 16 + (NB == 1 ? group >> 1 : group) * 8;
   const float cx = (float)gx + 3.5f, cy = (float)gy + 3.5f;  // its centre
-  const float xl = (float)(lane & 7) - 3.5f, yl = (float)(lane >> 3) - 3.5f;
-  const f2 YY = f2_pack(yl, yl + 4.f);
+  const float xl = (float)(gx + (lane & 7)), yl = (float)(gy + (lane >> 3));  // the lane's pixel of that block
   const uint2 rg = ranges[(size_t)b * T + tile];
   const float c2k = c2 * kNegHalfLog2e;
   float s[NB][2];
@@ -274,7 +262,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
     const float X = cx - ra.x, Y = cy - ra.y;
     const float lim = k0 + lane < rg.y ? rc.w : -1.f;  // num >= 0: no record meets nothing
     const float sy = __fdividef(-0.5f * ra.w, rb.x), sx = __fdividef(-0.5f * ra.w, ra.z);
-    const FwdScaled r = scale_record(ra, rb, rc);
+    const FwdEntry r = scale_record(ra, rb, rc);
     int cnt[NB];
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
@@ -288,7 +276,11 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
       const float Xq = X + (float)((q & 1) * 8), Yq = Y + (float)((q >> 1) * 8);
       const bool meets = ellipse_meets(ra.z, ra.w, rb.x, sx, sy, lim, Xq, Yq);
       const unsigned mask = __ballot_sync(0xffffffffu, meets);
-      if (meets) write_entry(r, Xq, Yq, &tables[warp][q][__popc(mask & ((1u << lane) - 1u)) * 3]);
+      if (meets) {
+        float4* e = &tables[warp][q][__popc(mask & ((1u << lane) - 1u)) * 3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) e[k] = r.q[k];
+      }
       cnt[q] = __popc(mask);
     }
     __syncwarp();
@@ -296,12 +288,14 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const float4* e = tables[warp][q];
+      const float x = xl + (float)((q & 1) * 8), y = yl + (float)((q >> 1) * 8);
+      const f2 YY = f2_pack(y, y + 4.f);
       // n entries from e: all evaluated (independent dependency chains), then accumulated in list order
       auto sweep = [&](int n) {
         FwdPair v[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (k < n) v[k] = fwd_pair(e + k * 3, xl, YY);
+          if (k < n) v[k] = fwd_pair(e + k * 3, x, YY);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (k < n) {
