@@ -260,13 +260,13 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
   if (first < rg.y) fetch(first);
   for (uint32_t k0 = first; k0 < rg.y; k0 += SP * C::batch) {
     const float X = cx - ra.x, Y = cy - ra.y;
-    const float lim = k0 + lane < rg.y ? rc.w : -1.f;  // num >= 0: no record meets nothing
+    const bool some = k0 + lane < rg.y;  // else the lane holds a record of the batch before, or none
     const float sy = __fdividef(-0.5f * ra.w, rb.x), sx = __fdividef(-0.5f * ra.w, ra.z);
     const FwdEntry r = scale_record(ra, rb, rc);
     int cnt[NB];
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
-      if (COUNT && lim >= 0.f) {
+      if (COUNT && some) {
         const int bx = __float_as_int(rc.y), by = __float_as_int(rc.z);
         const int qx = gx + (q & 1) * 8, qy = gy + (q >> 1) * 8;
         const int x0 = max(bx & 0xffff, qx), x1 = min(bx >> 16, qx + 7);
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
         if (x0 <= x1 && y0 <= y1) n_box += (unsigned)((x1 - x0 + 1) * (y1 - y0 + 1));
       }
       const float Xq = X + (float)((q & 1) * 8), Yq = Y + (float)((q >> 1) * 8);
-      const bool meets = ellipse_meets(ra.z, ra.w, rb.x, sx, sy, lim, Xq, Yq);
+      const bool meets = some && ellipse_meets(ra.z, ra.w, rb.x, sx, sy, rc.w, Xq, Yq);
       const unsigned mask = __ballot_sync(0xffffffffu, meets);
       if (meets) {
         float4* e = &tables[warp][q][__popc(mask & ((1u << lane) - 1u)) * 3];
