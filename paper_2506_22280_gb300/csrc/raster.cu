@@ -134,19 +134,25 @@ __device__ __forceinline__ HalfLanes group_lanes(int w, int h, int hl) {
 // ---- forward ------------------------------------------------------------------------------------
 
 // A CTA takes 16 x 16 pixels of a (projection, tile) (tiles of 32 pixels: four CTAs share a list), or a tile of
-// 8 x 8; tiles in the order `order` gives.  A warp owns NB of its 8 x 8 blocks and every SP-th batch of the
+// 8 x 8; tiles in the order `order` gives.  A warp owns `blocks` of its 8 x 8 blocks and every `splits`-th batch of the
 // list; lane l owns the pixels (l mod 8, l div 8) and (l mod 8, l div 8 + 4) of each block and keeps their sums
 // in registers.
-template <int TS, int NB, int SP>
+template <int TS>
 struct FwdCfg {
-  static constexpr int groups = TS == 8 ? 1 : 4 / NB;  // warps that share the CTA's blocks
-  static constexpr int warps = groups * SP;
+  static constexpr int blocks = TS == 8 ? 1 : 2;
+  static constexpr int groups = TS == 8 ? 1 : 4 / blocks;  // warps that share the CTA's blocks
+  // Four splits whatever the launch, so that a projection's sums, and its bits, do not depend on the views beside it.
+  // They cut the longest chain of work in launches of few CTAs (two against four splits: 16 views of 64^2 29 against
+  // 23 us); where a launch has many waves, two would do (a forward of 128 thorax projections, tiles of 8, 16 and 32
+  // pixels: 6.91, 6.06 and 6.41 ms with one or two splits, 7.08, 6.02 and 6.63 with four).
+  static constexpr int splits = 4;
+  static constexpr int warps = groups * splits;
   static constexpr int subs = TS == 32 ? 4 : 1;        // CTAs per tile
   static constexpr int threads = 32 * warps;
   static constexpr int batch = 32;                     // records a warp takes at a time: one per lane
-  // CTAs per SM that the registers are held to: 28 warps of 72 registers (NB = 1: 32 of 64).  For 128 thorax
-  // projections, 24, 28 and 32 warps took 4.41, 4.22 and 4.41 ms.
-  static constexpr int min_ctas = (NB == 1 ? 32 : 28) / warps;
+  static constexpr int step = splits * batch;          // from one of a warp's batches to its next
+  // CTAs per SM that the registers are held to: 24 warps of 80 registers (one block per warp: 32 of 64).
+  static constexpr int min_ctas = (blocks == 1 ? 32 : 24) / warps;
 };
 
 // A record as the pixel loops read it: with k = -log2(e) / 2 and sg = |amp| (1 when |amp| lies outside
@@ -219,16 +225,17 @@ __device__ __forceinline__ FwdPair fwd_pair(const float4* en, float x, f2 YY) {
 // that it meets; a ballot's prefix count gives the entry its place, packed and in list order, in the block's
 // table.  The warp then sweeps each block's table in order, four entries per step (independent dependency
 // chains, summed in list order): no canvas, no atomics, no CTA barrier.
-template <int TS, int NB, int SP, bool COUNT>
-__global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP>::min_ctas) k_raster_fwd(
+template <int TS, bool COUNT>
+__global__ void __launch_bounds__(FwdCfg<TS>::threads, FwdCfg<TS>::min_ctas) k_raster_fwd(
     const float4* __restrict__ grec, const uint32_t* __restrict__ srid, const uint2* __restrict__ ranges,
     const uint32_t* __restrict__ order, const __grid_constant__ ViewsParam views, int tiles_x, int T, int nu, int nv,
     float* __restrict__ proj, const float* __restrict__ meas, float* __restrict__ dldi,
     float* __restrict__ loss_part, float c2, float inv_count, unsigned long long* __restrict__ counters) {
-  using C = FwdCfg<TS, NB, SP>;
+  using C = FwdCfg<TS>;
+  constexpr int NB = C::blocks;
   __shared__ float4 tables[C::warps][NB][C::batch * 3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int group = SP == 1 ? warp : warp % C::groups, split = SP == 1 ? 0 : warp / C::groups;
+  const int group = warp % C::groups, split = warp / C::groups;
   const uint32_t bt = order[blockIdx.x / C::subs];  // heaviest (projection, tile) lists first
   const int sub = blockIdx.x % C::subs;
   const int b = (int)(bt / (uint32_t)T), tile = (int)(bt % (uint32_t)T);
@@ -254,11 +261,11 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
       rb = __ldg(src + 1);
       rc = __ldg(src + 2);
     }
-    const uint32_t kn = k0 + SP * C::batch + lane;
+    const uint32_t kn = k0 + C::step + lane;
     rid = kn < rg.y ? srid[kn] : 0u;
   };
   if (first < rg.y) fetch(first);
-  for (uint32_t k0 = first; k0 < rg.y; k0 += SP * C::batch) {
+  for (uint32_t k0 = first; k0 < rg.y; k0 += C::step) {
     const float X = cx - ra.x, Y = cy - ra.y;
     const bool some = k0 + lane < rg.y;  // else the lane holds a record of the batch before, or none
     const float sy = __fdividef(-0.5f * ra.w, rb.x), sx = __fdividef(-0.5f * ra.w, ra.z);
@@ -284,7 +291,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
       cnt[q] = __popc(mask);
     }
     __syncwarp();
-    fetch(k0 + SP * C::batch);  // arrives while this batch is swept
+    fetch(k0 + C::step);  // arrives while this batch is swept
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const float4* e = tables[warp][q];
@@ -314,7 +321,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
     }
     __syncwarp();
   }
-  if constexpr (SP > 1) {  // the splits' sums, added in split order by the first
+  {  // the splits' sums, added in split order by the first
     float* part = reinterpret_cast<float*>(&tables[0][0][0]);  // [warp][block][2][32]
     __syncthreads();
 #pragma unroll
@@ -327,7 +334,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
 #pragma unroll
       for (int q = 0; q < NB; ++q)
 #pragma unroll
-        for (int z = 1; z < SP; ++z) {
+        for (int z = 1; z < C::splits; ++z) {
           s[q][0] += part[(((z * C::groups + group) * NB + q) * 2) * 32 + lane];
           s[q][1] += part[(((z * C::groups + group) * NB + q) * 2 + 1) * 32 + lane];
         }
@@ -336,7 +343,7 @@ __global__ void __launch_bounds__(FwdCfg<TS, NB, SP>::threads, FwdCfg<TS, NB, SP
   const ViewC& v = views.v[b];
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
-    if (SP > 1 && split != 0) break;
+    if (split != 0) break;
     const int px = gx + (q & 1) * 8 + (lane & 7);
     float lsum = 0.f;
 #pragma unroll
@@ -594,17 +601,17 @@ __global__ void __launch_bounds__(256) k_gpix(const float* __restrict__ grad_pro
   gpix[idx] = grad_proj[idx] * pixel_ray_length(views.v[b], (float)(p % nu), (float)(p / nu));
 }
 
-template <int TS, int NB, int SP>
+template <int TS>
 static cudaError_t fwd_launch(const Workspace& ws, const ViewsParam& views, float c2, float* proj, const float* meas,
                               float* dldi, float inv_count, bool count, cudaStream_t st) {
-  using C = FwdCfg<TS, NB, SP>;
+  using C = FwdCfg<TS>;
   const unsigned grid = (unsigned)ws.T * (unsigned)ws.P * C::subs;
   float* lp = meas ? ws.loss_part : nullptr;
   if (count)
-    k_raster_fwd<TS, NB, SP, true><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
+    k_raster_fwd<TS, true><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
                                                         ws.nu, ws.nv, proj, meas, dldi, lp, c2, inv_count, ws.counters);
   else
-    k_raster_fwd<TS, NB, SP, false><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
+    k_raster_fwd<TS, false><<<grid, C::threads, 0, st>>>(ws.rec, ws.srid, ws.ranges, ws.order, views, ws.tiles_x, ws.T,
                                                          ws.nu, ws.nv, proj, meas, dldi, lp, c2, inv_count, ws.counters);
   note_launches(1);
   return cudaGetLastError();
@@ -614,25 +621,11 @@ cudaError_t launch_raster_fwd(const Workspace& ws, const ViewsParam& views, floa
                               float* dldi, float inv_count, cudaStream_t st) {
   if (ws.P <= 0) return cudaSuccess;
   const bool count = meas == nullptr;  // pair statistics are gathered by plain projections only
-  // How a tile's list is shared out (the sums differ only in rounding).  Splitting it over the CTA's warps cuts
-  // the longest chain of work; it costs a barrier and one more partly filled batch per split.  Four splits are
-  // the faster choice until the launch has a few waves of CTAs by itself (16-pixel tiles, two against four
-  // splits: 16 views of 64^2 0.029 / 0.023 ms, 4096 CTAs of the thorax 0.59 / 0.57, 8192 CTAs of 512^2
-  // 3.85 / 3.77, 10240 CTAs 1.34 / 1.36, 32768 CTAs 4.22 / 4.32; 8-pixel tiles, one against four: 16384 CTAs
-  // 0.59 / 0.56, 40960 CTAs 1.35 / 1.38; 32-pixel tiles, two against four: 10240 CTAs 1.62 / 1.59, 32768 equal).
-  const long long ctas = (long long)ws.P * ws.T * (ws.tile == 32 ? 4 : 1);
-  const bool few = ctas <= (ws.tile == 16 ? 8192 : 16384);
-#define DIGS_FWD(TS, NB, SP) return fwd_launch<TS, NB, SP>(ws, views, c2, proj, meas, dldi, inv_count, count, st)
+#define DIGS_FWD(TS) return fwd_launch<TS>(ws, views, c2, proj, meas, dldi, inv_count, count, st)
   switch (ws.tile) {
-    case 8:
-      if (few) DIGS_FWD(8, 1, 4);
-      DIGS_FWD(8, 1, 1);
-    case 16:
-      if (few) DIGS_FWD(16, 2, 4);
-      DIGS_FWD(16, 2, 2);
-    case 32:
-      if (few) DIGS_FWD(32, 2, 4);
-      DIGS_FWD(32, 2, 2);
+    case 8: DIGS_FWD(8);
+    case 16: DIGS_FWD(16);
+    case 32: DIGS_FWD(32);
   }
 #undef DIGS_FWD
   return cudaErrorInvalidValue;
