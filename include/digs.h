@@ -348,11 +348,12 @@ digs_status digs_gemm_bf16(int trans_a, int trans_b, int M, int N, int K, const 
                            int ldb, const float* bias, int relu, float* C, int ldc, int splits, float* partial,
                            int* status, void* stream);
 
-/* Tests each K-loop wait of digs_gemm_bf16's kernel makes on its mbarrier before it gives up (the
- * wait then sets *status to 1 and the output is undefined); tests < 0 restores the default (about
- * 4 x 10^6 tests, well under a second).  The final wait for the block's own tensor-core operations,
- * before it frees its tensor memory, always uses the default.  Process-wide; read when a GEMM is
- * launched (a captured graph keeps the value of its capture).  For testing the give-up path. */
+/* Tests each K-loop wait of a tensor-core kernel makes on its mbarrier before it gives up; tests < 0 restores the
+ * default (about 4 x 10^6 tests, well under a second).  A wait of digs_gemm_bf16's kernel that gives up sets *status
+ * to 1 and the output is undefined; one of the weight predictor's kernels makes the call's outputs that are computed
+ * after it NaN (the weights of a forward; the gradients of a backward, from that layer down).  The final wait for the
+ * block's own tensor-core operations and copies, before it leaves, always uses the default.  Process-wide; read when
+ * a kernel is launched (a captured graph keeps the value of its capture).  For testing the give-up path. */
 digs_status digs_set_wait_limit(long long tests);
 
 /* ---- Diagnostics (not part of the method; used to measure it) ---------------------------------- */

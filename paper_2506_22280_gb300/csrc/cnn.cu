@@ -141,7 +141,7 @@ __global__ void k_fc2_dh(const float* __restrict__ dout, const float* __restrict
   const int b = i / kHid, n = i - b * kHid;
   float s = 0.f;
   for (int r = 0; r < R; ++r) s = fmaf(dout[(size_t)b * R + r], w2[r * kHid + n], s);
-  const float v = h[i] > 0.f ? s : 0.f;
+  const float v = h[i] <= 0.f ? 0.f : s;  // h is NaN where its kernels gave up waiting: so is dh then
   dh[i] = v;
   if (dhb) dhb[i] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
 }

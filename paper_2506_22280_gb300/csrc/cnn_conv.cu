@@ -30,7 +30,7 @@
 // the same order as before.
 // One warp issues the copies, one the MMAs, four run the epilogue on the other half of the tensor memory; CTAs are
 // persistent, one per SM (layer 1's forward two: 411 -> 401 us a training step, 353 -> 343 the inference).  Every wait is bounded: a role that gives up sets *status, waits for what it has in
-// flight and leaves; the sums that follow turn into NaN (k_sum_z).
+// flight and leaves; the sums that follow are NaN (k_sum_z, k_colreduce_once).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -584,7 +584,7 @@ cudaError_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap
                    float* colpart, int tiles, int gx, int gy, unsigned* status, cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(k_conv<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<P>::kBytes);
   if (e != cudaSuccess) return e;
-  k_conv<P><<<dim3(gx, gy), kThreads, Smem<P>::kBytes, st>>>(a, b, io, out, bias, colpart, P::G::C, tiles, status, tc::kWaitLimit);
+  k_conv<P><<<dim3(gx, gy), kThreads, Smem<P>::kBytes, st>>>(a, b, io, out, bias, colpart, P::G::C, tiles, status, loop_wait_limit());
   note_launches(1);
   return cudaGetLastError();
 }
@@ -627,7 +627,7 @@ cudaError_t weight_gradient(const uint16_t* act, const uint16_t* dy, int B, floa
   const cudaError_t e = cudaFuncSetAttribute(k_conv_dw<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::kBytes);
   if (e != cudaSuccess) return e;
   const int n = (int)(px / 64);
-  k_conv_dw<L><<<dim3(P::kGroups, Z), kThreads, P::kBytes, st>>>(a, b, part, n, (n + Z - 1) / Z, status, tc::kWaitLimit);
+  k_conv_dw<L><<<dim3(P::kGroups, Z), kThreads, P::kBytes, st>>>(a, b, part, n, (n + Z - 1) / Z, status, loop_wait_limit());
   note_launches(1);
   return cudaGetLastError();
 }

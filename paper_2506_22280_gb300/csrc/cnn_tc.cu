@@ -11,8 +11,9 @@
 // mbarrier, and the accumulator goes through a per-role epilogue: feat W1^T (split K), the weight gradient
 // (transposed stores) and the data gradient (the last convolution's ReLU mask, its BF16 rounding and per-CTA column
 // sums for its bias gradient), the latter two with MN-major operands.
-// Every mbarrier wait is bounded; a K-loop wait that gives up sets *status and the CTA drains its own
-// MMAs (default bound) before it frees its tensor memory.
+// Every mbarrier wait is bounded; a K-loop wait that gives up sets *status, and the CTA drains its own MMAs (default
+// bound) and stores NaN for the tiles it owes before it frees its tensor memory.  Sums launched after that are NaN too
+// (k_sum_z, k_colreduce_once), so that nothing computed from a result that is missing looks like one.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -223,7 +224,7 @@ __device__ __forceinline__ uint64_t slice_desc(uint32_t a, int j) {
 // selects the stage buffer (g mod S) and the mbarrier phase (g div S).
 template <int BN, int kStages, bool AMN, bool BMN, class LA, class LB, class EP>
 __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2 ? 4 : (kStages == 3 ? 3 : 2)) : 1)) k_cnn_gemm(const LA la, const LB lb, const EP ep, int n_mt, int K, int kchunk,
-                                                      int* status, unsigned wait_limit, const void* any) {
+                                                      unsigned* status, unsigned wait_limit, const void* any) {
   using C = Cfg<BN, kStages>;
   extern __shared__ unsigned char smem_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -324,13 +325,24 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
     mt = next;
   }
   cp_wait<0>();
+  if (!ok) {  // the same for the whole CTA
+    for (; mt < n_mt; mt += gridDim.x)
+#pragma unroll 1
+      for (int c0 = 0; c0 < BN; c0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = __int_as_float(0x7fffffff);
+        float acc = 0.f;
+        ep.apply(mt * kBM + warp * 32 + lane, n0 + c0, v, acc, scratch);
+      }
+    if (tid == 0) atomicExch(status, 1u);
+  }
   tc::fence_before();
   __syncthreads();
   if (warp == 0) {
     tc::fence_after();
     tc::tmem_dealloc(tmem, BN);
   }
-  if (!ok && tid == 0 && status) atomicExch(status, 1);
 }
 
 // ---- SIMT kernels and small steps --------------------------------------------------------------------
@@ -553,7 +565,7 @@ __global__ void __launch_bounds__(256, 2) k_conv0_dw(const T* __restrict__ dy, c
 // on which block finishes last, and no block waits for another.
 __global__ void __launch_bounds__(256) k_colreduce_once(const float* __restrict__ in, int R, int cols, int ld,
                                                         int chunk, float* part, float* __restrict__ out,
-                                                        unsigned* tickets) {
+                                                        unsigned* tickets, const unsigned* status) {
   __shared__ float red[8][32];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -585,6 +597,7 @@ __global__ void __launch_bounds__(256) k_colreduce_once(const float* __restrict_
     float t = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) t += red[k][lane];
+    if (status && *status) t = __int_as_float(0x7fffffff);
     out[c] = t;
   }
   if (threadIdx.x == 0) tickets[blockIdx.x] = 0u;
@@ -670,7 +683,7 @@ unsigned grid_of(long long n) { return (unsigned)std::max<long long>(1, std::min
 // One GEMM launch: M rows of C in 128-row tiles, gy column tiles of BN, gz splits (or classes).
 template <int BN, int S, bool AMN, bool BMN, class LA, class LB, class EP>
 cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy, int gz, int kchunk, const void* any,
-                 cudaStream_t st) {
+                 unsigned* status, cudaStream_t st) {
   using C = Cfg<BN, S>;
   auto kern = k_cnn_gemm<BN, S, AMN, BMN, LA, LB, EP>;
   static bool configured = false;
@@ -687,7 +700,7 @@ cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy,
   const long long total = (long long)n_mt * gy * gz, target = 4LL * 152 * per_sm;
   const int per_cta = (int)std::max(1LL, (total + target - 1) / target);
   const int gx = (n_mt + per_cta - 1) / per_cta;
-  kern<<<dim3(gx, gy, gz), kThr, C::kSmem, st>>>(la, lb, ep, n_mt, K, kchunk, nullptr, tc::kWaitLimit, any);
+  kern<<<dim3(gx, gy, gz), kThr, C::kSmem, st>>>(la, lb, ep, n_mt, K, kchunk, status, loop_wait_limit(), any);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -707,11 +720,11 @@ int chunk_of(long long n, int z) { return (int)(((n + z - 1) / z + kBK - 1) / kB
 // many blocks, then the chunk sums by one block per 32 columns (one pass when R <= 512).
 // tickets: (cols + 31) / 32 counters, zero on entry (and left zero).
 cudaError_t colreduce(const float* in, int R, int cols, int ld, float* out, float* scratch, unsigned* tickets,
-                      cudaStream_t st) {
+                      const unsigned* status, cudaStream_t st) {
   const unsigned gx = (unsigned)((cols + 31) / 32);
   // at most 512 chunks: the last block adds their sums one after the other
   const int chunk = R <= 2048 ? 64 : std::max(128, (R + 511) / 512), nch = (R + chunk - 1) / chunk;
-  k_colreduce_once<<<dim3(gx, nch), 256, 0, st>>>(in, R, cols, ld, chunk, scratch, out, tickets);
+  k_colreduce_once<<<dim3(gx, nch), 256, 0, st>>>(in, R, cols, ld, chunk, scratch, out, tickets, status);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -719,11 +732,11 @@ cudaError_t colreduce(const float* in, int R, int cols, int ld, float* out, floa
 // dW of the first convolution into out (32 x 9): at most kConv0Ctas partial sums in colpart, then added.
 template <typename T>
 cudaError_t conv0_dw(const T* dy, const T* img, int B, float* colpart, float* scratch, unsigned* tickets, float* out,
-                     cudaStream_t st) {
+                     const unsigned* status, cudaStream_t st) {
   const int ctas = std::min(kConv0Ctas, B * kBands);
   k_conv0_dw<T><<<ctas, 256, 0, st>>>(dy, img, B * kBands, colpart);
   note_launches(1);
-  return colreduce(colpart, ctas, 288, 288, out, scratch, tickets, st);
+  return colreduce(colpart, ctas, 288, 288, out, scratch, tickets, status, st);
 }
 
 }  // namespace
@@ -796,7 +809,7 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
   const int Z = 16, kc = chunk_of(kFeatPitch, Z);
   const EpiF32 ep{t.part, (long long)B * kHid, B, kHid};
   TC_TRY((gemm<128, 4, false, false>(PlainK{(const bf16*)t.feat, kFeatPitch, B}, PlainK{(const bf16*)t.w1b, kFeatPitch, kHid},
-                                  ep, B, kFeatPitch, 1, Z, kc, any, st)));
+                                  ep, B, kFeatPitch, 1, Z, kc, any, t.status, st)));
   k_sum_z<<<(unsigned)(((long long)B * kHid + 31) / 32), 256, 0, st>>>(t.part, Z, (long long)B * kHid, net.b1, kHid, h, t.status);
   note_launches(1);
   return cudaGetLastError();
@@ -809,14 +822,14 @@ cudaError_t cnn_tc_backward(int B, const CnnTc& t, const float* dh, const CnnGra
   if (ez != cudaSuccess) return ez;
   // dense layer: dW1[n][f] = sum_b dh[b][n] feat[b][f] (rows f, both operands MN-major)
   TC_TRY((gemm<128, 3, true, true>(PlainMN{(const bf16*)t.feat, kFeatPitch, kFeatPitch}, PlainMN{(const bf16*)t.dhb, kHid, kHid},
-                                EpiF32T{g.w1, 0, kFeat + 2, kFeat + 2}, kFeatPitch, B, 1, 1, B, any, st)));
+                                EpiF32T{g.w1, 0, kFeat + 2, kFeat + 2}, kFeatPitch, B, 1, 1, B, any, t.status, st)));
   // ... and dfeat[b][f] = sum_n dh[b][n] W1[n][f] (rows b, B MN-major) -> dY of the last convolution
   // (masked, BF16) and its per-channel column sums
   const int nmt = (B + kBM - 1) / kBM;
   TC_TRY((gemm<128, 2, false, true>(PlainK{(const bf16*)t.dhb, kHid, B}, PlainMN{(const bf16*)t.w1b, kFeatPitch, kFeat},
                                     EpiDfeat{(bf16*)t.dy3, (const bf16*)t.feat, t.colpart, B}, B, kHid, kFeat / 128, 1,
-                                    kHid, any, st)));
-  TC_TRY(colreduce(t.colpart, (kFeat / 128) * nmt, 128, 128, g.b[3], t.part, t.tickets, st));
+                                    kHid, any, t.status, st)));
+  TC_TRY(colreduce(t.colpart, (kFeat / 128) * nmt, 128, 128, g.b[3], t.part, t.tickets, t.status, st));
   // convolutions 3, 2, 1: weight gradient (split over pixels), then the data gradient of the layer below
   const uint16_t* dyl = t.dy3;
   for (int l = 3; l >= 1; --l) {
@@ -828,22 +841,22 @@ cudaError_t cnn_tc_backward(int B, const CnnTc& t, const float* dh, const CnnGra
     // output dY of convolution l - 1 and its bias partials, a row per CTA
     uint16_t* dyo = l == 2 ? t.dy[1] : t.dy[0];
     TC_TRY(cnn_conv_dx(l, dyl, t.wt[l], t.act[l - 1], B, dyo, t.colpart, t.status, st));
-    TC_TRY(colreduce(t.colpart, cnn_conv_dx_rows(l, B), kCh[l], kCh[l], g.b[l - 1], t.part, t.tickets, st));
+    TC_TRY(colreduce(t.colpart, cnn_conv_dx_rows(l, B), kCh[l], kCh[l], g.b[l - 1], t.part, t.tickets, t.status, st));
     dyl = dyo;
   }
   // the first convolution's weight gradient on the SIMT pipes
-  TC_TRY(conv0_dw((const bf16*)dyl, (const bf16*)t.imgb, B, t.colpart, t.part, t.tickets, g.w[0], st));
+  TC_TRY(conv0_dw((const bf16*)dyl, (const bf16*)t.imgb, B, t.colpart, t.part, t.tickets, g.w[0], t.status, st));
   return cudaGetLastError();
 }
 
 cudaError_t cnn_colsum(const float* dY, int M, int N, const CnnTc& t, float* out, cudaStream_t st) {
   const cudaError_t e = cudaMemsetAsync(t.tickets, 0, kColTickets * sizeof(unsigned), st);
-  return e != cudaSuccess ? e : colreduce(dY, M, N, N, out, t.part, t.tickets, st);
+  return e != cudaSuccess ? e : colreduce(dY, M, N, N, out, t.part, t.tickets, nullptr, st);
 }
 
 cudaError_t cnn_conv0_dw_f32(const float* dy, const float* img, int B, const CnnTc& t, float* out, cudaStream_t st) {
   const cudaError_t e = cudaMemsetAsync(t.tickets, 0, kColTickets * sizeof(unsigned), st);
-  return e != cudaSuccess ? e : conv0_dw(dy, img, B, t.colpart, t.part, t.tickets, out, st);
+  return e != cudaSuccess ? e : conv0_dw(dy, img, B, t.colpart, t.part, t.tickets, out, nullptr, st);
 }
 
 cudaError_t cnn_sum_splits(const float* part, int Z, long long n, const float* bias, int nb, float* out, cudaStream_t st) {

@@ -10,6 +10,8 @@ namespace digs {
 
 // Kernel-launch bookkeeping (diagnostic): every launcher reports how many kernels it enqueued.
 void note_launches(int k);
+// Tests a tensor-core kernel's mbarrier wait makes before it gives up (umma.cu: digs_set_wait_limit).
+unsigned loop_wait_limit();
 
 // Workspace carve-up for one call.  Every pointer is 256-byte aligned inside the caller's buffer.
 struct Workspace {
@@ -145,7 +147,7 @@ struct CnnTc {
   float *part, *colpart;
   long long part_floats, colpart_floats;
   unsigned* tickets;  // counters of the single-launch column reductions (zeroed by cnn_tc_backward)
-  unsigned* status;   // zeroed by cnn_tc_forward; set by a convolution kernel that gave up waiting
+  unsigned* status;   // zeroed by cnn_tc_forward; set by a kernel that gave up waiting: the sums that follow are NaN
 };
 // Bytes of the buffers for batch B (base == nullptr: size only), 256-byte aligned.
 size_t cnn_tc_layout(void* base, int B, CnnTc* t);

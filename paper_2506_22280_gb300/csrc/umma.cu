@@ -291,6 +291,8 @@ cudaError_t gemm_tc_sum(bool at, bool bt, int M, int N, int K, const float* A, i
   return cudaGetLastError();
 }
 
+unsigned loop_wait_limit() { return g_loop_wait_limit; }
+
 }  // namespace digs
 
 extern "C" digs_status digs_set_wait_limit(long long tests) {

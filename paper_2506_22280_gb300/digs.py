@@ -166,7 +166,7 @@ def pipe_rate(kind: str, iters: int = 4096, reps: int = 3) -> float:
 
 
 def set_wait_limit(tests: int) -> None:
-    """Tests a tensor-core GEMM K-loop wait makes before it gives up (< 0: the default)."""
+    """Tests a wait of a tensor-core kernel's K loop makes before it gives up (< 0: the default)."""
     _check(lib().digs_set_wait_limit(int(tests)), "digs_set_wait_limit")
 
 
