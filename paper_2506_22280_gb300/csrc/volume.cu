@@ -29,9 +29,14 @@ struct GridC {
 // 100k Gaussians into 128^3 voxels of 2 mm: 2.22 -> 0.22 ms.
 constexpr int kVoxWarps = 4;
 
-__device__ __forceinline__ float exp2_sfu(float x) {  // flushes subnormals: e^(-E/2) there is below 1.2e-38
+// 2^x by the SFU; SUB: with subnormal results, which cost instructions and come up beyond E = 2 ln 2^126 only.
+template <bool SUB>
+__device__ __forceinline__ float exp2_sfu(float x) {
   float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  if (SUB)
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  else
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 // *p += v where E <= c2, without a branch around the one instruction.
@@ -46,7 +51,11 @@ struct VoxRec {
   int lo[3], ext[3];  // ext[0] = 0: nothing to add
 };
 
-template <int R>
+// WIDE: cutoffs whose values reach below 2^-126 and grids of more than 2^24 layers (layer numbers no longer exact in
+// FP32); otherwise z is counted in FP32, one conversion per voxel fewer.
+constexpr float kWideC2 = 174.f;  // 2 ln 2^126 = 174.67, with room for rounding
+constexpr int kWideLayers = 1 << 24;
+template <int R, bool WIDE>
 __global__ void __launch_bounds__(32 * kVoxWarps) k_voxelize(GaussPtrs g, LatticeC L, const float* __restrict__ phi,
                                                              const float* __restrict__ w, GridC G, float c2,
                                                              float* __restrict__ vol) {
@@ -133,19 +142,20 @@ __global__ void __launch_bounds__(32 * kVoxWarps) k_voxelize(GaussPtrs g, Lattic
     const size_t plane = (size_t)G.ny * G.nx;
     const int sy = 32 / ex, sx = 32 - sy * ex;  // a step of 32 columns (x, y), x fastest
     int y = lane / ex, x = lane - y * ex;
-    for (int c0 = 0; c0 < ex * ey; c0 += 32) {
+    const unsigned steps = (unsigned)(((long long)ex * ey + 31) >> 5);
+    for (unsigned c0 = 0; c0 < steps; ++c0) {
       if (y < ey) {
         const int i = r.lo[0] + x, j = r.lo[1] + y;
         const float dx = G.origin[0] + i * G.spacing[0] - mx;
         const float dy = G.origin[1] + j * G.spacing[1] - my;
         float* p = vol + ((size_t)r.lo[2] * G.ny + j) * G.nx + i;
-        float k = (float)r.lo[2];  // whole numbers: exact
+        float k = (float)r.lo[2];
 #pragma unroll 4
-        for (int z = 0; z < ez; ++z, p += plane, k += 1.f) {
+        for (int z = 0; z < ez; ++z, p += plane, k = WIDE ? (float)(r.lo[2] + z) : k + 1.f) {
           const float dz = G.origin[2] + k * G.spacing[2] - mz;
           const float E = r.P[0] * dx * dx + r.P[1] * dy * dy + r.P[2] * dz * dz +
                           2.f * (r.P[3] * dx * dy + r.P[4] * dx * dz + r.P[5] * dy * dz);
-          add_within(p, rho * exp2_sfu(-0.5f * E * DIGS_LOG2E), E, c2);
+          add_within(p, rho * exp2_sfu<WIDE>(-0.5f * E * DIGS_LOG2E), E, c2);
         }
       }
       x += sx;
@@ -323,12 +333,17 @@ digs_status digs_voxelize(const DigsGaussians* g, const DigsLattice* lat, const 
   if (g->n == 0) return DIGS_OK;
   GaussPtrs gp{g->mu0, g->scale, g->quat, g->rho, g->n};
   const unsigned blocks = (unsigned)((g->n + 31LL) / 32);
+  const bool wide = cut * cut > kWideC2 || G.nz > kWideLayers;
+#define DIGS_VOX(RR)                                                                              \
+  if (wide) k_voxelize<RR, true><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol); \
+  else k_voxelize<RR, false><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol)
   switch (L.R) {
-    case 1: k_voxelize<1><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol); break;
-    case 2: k_voxelize<2><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol); break;
-    case 3: k_voxelize<3><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol); break;
-    case 4: k_voxelize<4><<<blocks, 32 * kVoxWarps, 0, st>>>(gp, L, phi, w, G, cut * cut, vol); break;
+    case 1: DIGS_VOX(1); break;
+    case 2: DIGS_VOX(2); break;
+    case 3: DIGS_VOX(3); break;
+    case 4: DIGS_VOX(4); break;
   }
+#undef DIGS_VOX
   note_launches(1);
   return cudaGetLastError() == cudaSuccess ? DIGS_OK : DIGS_ERR_CUDA;
 }
