@@ -201,19 +201,21 @@ __device__ __forceinline__ void pair_adjoint(const ViewC& v, const float* __rest
   inv3(K, Ki);
   make_A(inv_s, Rm, Ki, A);
   float gA[9];
-  // The ten sums of the record's gradient from its pixel moments M (see bwd_box_pixels): with B = A (E - 1) its
-  // moments b = M[6..] / k - M[0..], t = 1 + u x + v y (u = wn0, v = wn1) and num = p x^2 + q x y + r y^2,
-  // S[0] = sum g V / amp = sum A D, S[1..5] = sum dL/dnum (x^2, x y, y^2, x, y), S[6..8] = sum dL/dt (1, x, y),
-  // S[9] = sum dL/dkappa.
+  // The ten sums of the record's gradient from its pixel moments M (see bwd_box_pixels): with t = 1 + u x + v y
+  // (u = wn0, v = wn1) and num = p x^2 + q x y + r y^2, S[0] = sum g V / amp = sum A D, where D = t^2 + kap num gives
+  // sum A; with B = A (E - 1) its moments b = M[6..] / k - (sum A, M[1..5]); S[1..5] = sum dL/dnum (x^2, x y, y^2, x, y),
+  // S[6..8] = sum dL/dt (1, x, y), S[9] = sum dL/dkappa.
   float S[10];
   auto record_sums = [&](float u, float v, float kap, float p, float q, float r, float amp) {
     constexpr float ik = -2.f / DIGS_LOG2E;
+    const float a0 = M[0] - (2.f * (u * M[1] + v * M[3]) + (u * u + kap * p) * M[2] + (2.f * u * v + kap * q) * M[4] +
+                             (v * v + kap * r) * M[5]);
     float b[6];
+    b[0] = fmaf(ik, M[6], -a0);
 #pragma unroll
-    for (int j = 0; j < 6; ++j) b[j] = fmaf(ik, M[6 + j], -M[j]);
+    for (int j = 1; j < 6; ++j) b[j] = fmaf(ik, M[6 + j], -M[j]);
     const float h = 0.5f * amp;
-    S[0] = M[0] + 2.f * (u * M[1] + v * M[3]) + (u * u + kap * p) * M[2] + (2.f * u * v + kap * q) * M[4] +
-           (v * v + kap * r) * M[5];
+    S[0] = M[0];
     S[1] = h * fmaf(kap, b[2], -M[2]);
     S[2] = h * fmaf(kap, b[4], -M[4]);
     S[3] = h * fmaf(kap, b[5], -M[5]);

@@ -384,14 +384,16 @@ __global__ void __launch_bounds__(FwdCfg<TS>::threads, FwdCfg<TS>::min_ctas) k_r
 
 
 // Adds the lane's share of a record's twelve pixel moments: with A = (g V / amp) / D and k E the exp2 argument,
-//   Sv[0..5] = sum A (1, dx, dx^2, dy, dx dy, dy^2) and Sv[6..11] = sum A k E (the same),
+//   Sv[0] = sum g V / amp, Sv[1..5] = sum A (dx, dx^2, dy, dx dy, dy^2) and Sv[6..11] = sum A k E (1, dx, dx^2, dy, ...),
 // (dx, dy) the pixel's offset from the projected mean.  With B = A (E - 1): dL/dnum = (amp / 2) (kappa B - A),
 // dL/dt = amp B t, dL/dkappa = (amp / 2) B num and g V / amp = A D, and t, num and D are polynomials of degree two
-// in (dx, dy), so the ten sums of the record's gradient follow from these twelve with per-record constants:
-// pair_adjoint forms them, once per record, instead of every lane of the sweep once per slice of the box.
+// in (dx, dy), so the ten sums of the record's gradient and sum A follow from these twelve with per-record constants:
+// pair_adjoint forms them, once per record, instead of every lane of the sweep once per slice of the box.  (The density's
+// gradient is Sv[0] alone.  Taken from sum A and the others it costs an addition per pair fewer, 3 %, and carries the
+// rounding of 1 / D and back: 3.7 % further from FP64 in the thorax's steps.)
 // gp points at g = dL/dI * |X - s| of the lane's first pixel in the projection image (row pitch nu); (dx1, dy1)
-// is that pixel's offset.  A lane's pixel keeps its column, so the loop accumulates the six dy-moments alone (20
-// packed operations per pixel pair, 23 with the seven sums it kept before).
+// is that pixel's offset.  A lane's pixel keeps its column, so the loop accumulates the six dy-moments and sum g V / amp
+// alone (21 packed operations per pixel pair).
 __device__ __forceinline__ void bwd_box_pixels(const Rec& R0, const HalfLanes& B, int h, float dx1, float dy1,
                                                const float* __restrict__ gp, int nu, float c2, float Sv[12]) {
   // k = -log2(e) / 2 is folded into the quadratic form: NUM = k num, ARG = k E (the exp2 argument)
@@ -404,7 +406,7 @@ __device__ __forceinline__ void bwd_box_pixels(const Rec& R0, const HalfLanes& B
   const f2 C2K = f2_dup(c2 * kNegHalfLog2e);
   const int pstep = B.ystep * nu, d2 = B.pdy * nu + B.pdx, hb = B.col2 ? h - B.pdy : 0;
   f2 DY = f2_pack(dy1, dy1 + (float)B.pdy);
-  f2 A0 = f2_dup(0.f), A1 = A0, A2 = A0, E0 = A0, E1 = A0, E2 = A0;
+  f2 G0 = f2_dup(0.f), A0 = G0, A1 = G0, A2 = G0, E0 = G0, E1 = G0, E2 = G0;
   for (int r = B.r0; r < h; r += B.ystep, DY = f2_add(DY, STEP), gp += pstep) {
     const f2 NUM = f2_fma(DY, f2_fma(N11, DY, BQ), AQ);
     const f2 T = f2_fma(WN1, DY, T0);
@@ -421,9 +423,11 @@ __device__ __forceinline__ void bwd_box_pixels(const Rec& R0, const HalfLanes& B
     const f2 INVD = f2_mul(RS, RS);
     const f2 ARG = f2_mul(NUM, INVD);
     const f2 BV = f2_mul(RS, f2_exp2(ARG));                            // V / amp
-    const f2 AL = f2_mul(f2_mul(f2_pack(ga, gb), BV), INVD);           // A
+    const f2 GA = f2_mul(f2_pack(ga, gb), BV);                         // g V / amp
+    const f2 AL = f2_mul(GA, INVD);                                    // A
     const f2 AE = f2_mul(AL, ARG);                                     // A k E
     const f2 DY2 = f2_mul(DY, DY);
+    G0 = f2_add(G0, GA);
     A0 = f2_add(A0, AL);
     A1 = f2_fma(AL, DY, A1);
     A2 = f2_fma(AL, DY2, A2);
@@ -437,7 +441,7 @@ __device__ __forceinline__ void bwd_box_pixels(const Rec& R0, const HalfLanes& B
     Sv[q] += lo + hi;
   };
   const f2 AX = f2_mul(A0, DX), EX = f2_mul(E0, DX);
-  add(0, A0);
+  add(0, G0);
   add(1, AX);
   add(2, f2_mul(AX, DX));
   add(3, A1);
