@@ -155,7 +155,8 @@ long long capacity_for(size_t bytes, int n, int P, int nu, int nv, int R, int ti
     long long mid = (lo + hi) / 2;
     if (layout(nullptr, nullptr, n, P, nu, nv, R, mid, tile, n_total, w_rows) <= bytes) lo = mid; else hi = mid;
   }
-  return std::min(lo, (long long)0xffffffffLL);
+  // pair numbers are 32 bits wide, and the rasters' loops run up to a few batches past a list's end
+  return std::min(lo, (1LL << 32) - 4096);
 }
 
 size_t phi_floats(const LatticeC& L) { return (size_t)L.nx * L.ny * L.nz * 3 * L.R; }
