@@ -6,15 +6,15 @@
 // Network: four 3 x 3 convolutions of stride 2 and padding 1 (1 -> 32 -> 64 -> 128 -> 128 channels,
 // 128^2 -> 64^2 -> 32^2 -> 16^2 -> 8^2), each followed by ReLU; the 8 x 8 x 128 features and
 // (cos theta, sin theta) feed a 128-unit ReLU layer and a linear layer to R outputs.  Activations are
-// NHWC; a convolution is im2col (rows = output pixels, columns = (ky, kx, c)) times the transposed
-// weight matrix W[Co][ky][kx][Ci], so every layer, forward and backward, is one of three GEMM forms:
+// NHWC.  With rows = output pixels and columns = (ky, kx, c) of the inputs they read, a convolution is a product with
+// the transposed weight matrix W[Co][ky][kx][Ci], and every layer, forward and backward, one of three forms:
 //   forward      Y[M][N]  = X[M][K] W[N][K]^T      (+ bias, ReLU)
 //   data grad    dX[M][K] = dY[M][N] W[N][K]
 //   weight grad  dW[N][K] = dY[M][N]^T X[M][K]     (split over M, partials summed in a fixed order)
-// The forward and backward run either in FP32 on the SIMT pipes or, with DIGS_CNN_TENSOR_CORES, with the
-// large GEMMs (the convolutions but the first, and the 8194-wide layer) on the tensor cores: BF16 operands rounded from
-// the FP32 activations, gradients and weights, FP32 accumulation; the R-wide output layer stays FP32.
-// Inference reads BF16 weights and activations and runs its large GEMMs on the tensor cores.
+// X is read in place, never written out.  The forward and backward run either in FP32 on the SIMT pipes (cnn_f32.cu)
+// or, with DIGS_CNN_TENSOR_CORES, with the large products (the convolutions but the first, and the 8194-wide layer)
+// on the tensor cores (cnn_tc.cu, cnn_conv.cu): BF16 activations, gradients and weights, FP32 accumulation; the R-wide
+// output layer stays FP32.  Inference runs the tensor-core forward.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -27,7 +27,6 @@ namespace {
 
 constexpr int kConvs = 4;
 constexpr int kCh[kConvs + 1] = {1, 32, 64, 128, 128};
-constexpr int kEdge[kConvs + 1] = {128, 64, 32, 16, 8};
 constexpr int kFeat = 8 * 8 * 128;
 constexpr int kFeatIn = kFeat + 2;
 constexpr int kHid = 128;
@@ -59,7 +58,6 @@ ParamOffsets param_offsets(int R) {
   return o;
 }
 
-size_t rows(int l, int B) { return (size_t)B * kEdge[l + 1] * kEdge[l + 1]; }  // output pixels of conv l
 size_t kdim(int l) { return (size_t)9 * kCh[l]; }
 
 // Workspace of one batch: activations for the backward, gradients, split-K partials, BF16 copies.
@@ -210,23 +208,20 @@ __global__ void k_init(float* __restrict__ p, long long n, unsigned long long se
   }
 }
 
-template <typename T>
-struct NetPtrs {  // one precision's view of the parameters
-  const T *w[kConvs], *w1, *w2;
-  const float *b[kConvs], *b1, *b2;
+struct NetPtrs {
+  const float *w[kConvs], *b[kConvs], *w1, *b1, *w2, *b2;
 };
 
-template <typename T>
-NetPtrs<T> net_ptrs(const T* wp, const float* bp, const ParamOffsets& o) {
-  NetPtrs<T> n;
+NetPtrs net_ptrs(const float* p, const ParamOffsets& o) {
+  NetPtrs n;
   for (int l = 0; l < kConvs; ++l) {
-    n.w[l] = wp + o.w[l];
-    n.b[l] = bp + o.b[l];
+    n.w[l] = p + o.w[l];
+    n.b[l] = p + o.b[l];
   }
-  n.w1 = wp + o.w1;
-  n.b1 = bp + o.b1;
-  n.w2 = wp + o.w2;
-  n.b2 = bp + o.b2;
+  n.w1 = p + o.w1;
+  n.b1 = p + o.b1;
+  n.w2 = p + o.w2;
+  n.b2 = p + o.b2;
   return n;
 }
 
@@ -236,7 +231,7 @@ NetPtrs<T> net_ptrs(const T* wp, const float* bp, const ParamOffsets& o) {
     if (e__ != cudaSuccess) return e__;      \
   } while (0)
 
-CnnNet cnn_net(const NetPtrs<float>& N) {
+CnnNet cnn_net(const NetPtrs& N) {
   CnnNet n;
   for (int l = 0; l < kConvs; ++l) {
     n.w[l] = N.w[l];
@@ -250,7 +245,7 @@ CnnNet cnn_net(const NetPtrs<float>& N) {
 // Forward keeping every activation in the workspace for the backward.  tc: the tensor-core path of
 // cnn_tc.cu up to the dense layer's output (BF16 activations), else the FP32 SIMT GEMMs of cnn_f32.cu; the
 // R-wide output layer is FP32 either way.
-cudaError_t forward_f32(const NetPtrs<float>& N, int R, const float* img, const float* cs, int B, const CnnWs& w,
+cudaError_t forward_f32(const NetPtrs& N, int R, const float* img, const float* cs, int B, const CnnWs& w,
                         bool tc, cudaStream_t st) {
   if (tc) {
     CNN_TRY(cnn_tc_forward(cnn_net(N), img, cs, B, w.tc, w.h, st));
@@ -263,7 +258,7 @@ cudaError_t forward_f32(const NetPtrs<float>& N, int R, const float* img, const 
 }
 
 // Backward of forward_f32 for dL/dout in w.dout; writes every parameter gradient to grad (layout as params).
-cudaError_t backward_f32(const NetPtrs<float>& N, const ParamOffsets& o, int R, int B, const CnnWs& w, float* grad,
+cudaError_t backward_f32(const NetPtrs& N, const ParamOffsets& o, int R, int B, const CnnWs& w, float* grad,
                          bool tc, cudaStream_t st) {
   // output layer
   k_fc2_wgrad<<<kFc2Blocks, kHid + 32, 0, st>>>(w.dout, w.h, B, R, w.part);
@@ -327,7 +322,7 @@ digs_status digs_cnn_forward(const float* params, int R, const float* img, const
   const ParamOffsets o = param_offsets(R);
   cudaStream_t st = (cudaStream_t)stream;
   const bool tc = (flags & DIGS_CNN_TENSOR_CORES) != 0;
-  if (forward_f32(net_ptrs<float>(params, params, o), R, img, cs, B, w, tc, st) != cudaSuccess) return DIGS_ERR_CUDA;
+  if (forward_f32(net_ptrs(params, o), R, img, cs, B, w, tc, st) != cudaSuccess) return DIGS_ERR_CUDA;
   if (cudaMemcpyAsync(w_out, w.out, (size_t)B * R * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return DIGS_ERR_CUDA;
   return DIGS_OK;
@@ -343,7 +338,7 @@ digs_status digs_cnn_backward(const float* params, int R, int B, const float* gr
   if (cudaMemcpyAsync(w.dout, grad_w, (size_t)B * R * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return DIGS_ERR_CUDA;
   const bool tc = (flags & DIGS_CNN_TENSOR_CORES) != 0;
-  if (backward_f32(net_ptrs<float>(params, params, o), o, R, B, w, grad_params, tc, st) != cudaSuccess)
+  if (backward_f32(net_ptrs(params, o), o, R, B, w, grad_params, tc, st) != cudaSuccess)
     return DIGS_ERR_CUDA;
   return DIGS_OK;
 }
@@ -357,7 +352,7 @@ digs_status digs_cnn_train_step(float* params, float* m, float* v, float* grad, 
   if (w.bytes > ws_bytes) return DIGS_ERR_ARG;
   const ParamOffsets o = param_offsets(R);
   cudaStream_t st = (cudaStream_t)stream;
-  const NetPtrs<float> N = net_ptrs<float>(params, params, o);
+  const NetPtrs N = net_ptrs(params, o);
   const bool tc = (flags & DIGS_CNN_TENSOR_CORES) != 0;
   if (forward_f32(N, R, img, cs, B, w, tc, st) != cudaSuccess) return DIGS_ERR_CUDA;
   k_mse<<<1, 256, 0, st>>>(w.out, target, B * R, w.dout, loss_out);
@@ -375,7 +370,7 @@ digs_status digs_cnn_infer_bf16(const float* params, int R, const float* img, co
   if (w.bytes > ws_bytes) return DIGS_ERR_ARG;
   const ParamOffsets o = param_offsets(R);
   cudaStream_t st = (cudaStream_t)stream;
-  const NetPtrs<float> N = net_ptrs<float>(params, params, o);
+  const NetPtrs N = net_ptrs(params, o);
   if (cnn_tc_forward(cnn_net(N), img, cs, B, w.tc, w.h, st) != cudaSuccess) return DIGS_ERR_CUDA;
   k_fc2_fwd<<<(B + 7) / 8, 256, 0, st>>>(w.h, N.w2, N.b2, B, R, w_out);
   note_launches(1);

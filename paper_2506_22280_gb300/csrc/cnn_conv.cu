@@ -188,7 +188,7 @@ struct Fwd {
 };
 
 // ---- data gradient ------------------------------------------------------------------------------------
-// blockIdx.y selects CC of the C input channels.  Weights: rows of 64 output channels, see cnn_conv_wt.
+// blockIdx.y selects CC of the C input channels.  Weights: rows of 64 output channels, as k_to_bf16_jobs lays them out (kind 1).
 template <int L>
 struct Dx {
   using G = Geo<L>;

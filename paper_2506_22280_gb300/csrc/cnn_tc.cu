@@ -7,7 +7,7 @@
 // has a single input channel (K = 9) and runs on the SIMT pipes with the same rounded operands.  The dense layer's
 // three GEMMs are launches of one kernel template: 128 threads per CTA, looping over 128-row tiles of C; the four
 // warps fill a ring of 2-4 stages of 64-deep K slices of A and B with 16-byte cp.async copies (zero-filled where an
-// operand is padding), one thread issues the four 128 x BN x 16 MMAs of a slice and commits them to the slice's
+// operand is padding), one thread issues the four 128 x 128 x 16 MMAs of a slice and commits them to the slice's
 // mbarrier, and the accumulator goes through a per-role epilogue: feat W1^T (split K), the weight gradient
 // (transposed stores) and the data gradient (the last convolution's ReLU mask, its BF16 rounding and per-CTA column
 // sums for its bias gradient), the latter two with MN-major operands.
@@ -27,7 +27,7 @@ namespace {
 typedef __nv_bfloat16 bf16;
 
 constexpr int kThr = 128;
-constexpr int kBM = 128, kBK = 64;
+constexpr int kBM = 128, kBN = 128, kBK = 64;
 
 // ---- geometry of the network (cnn.cu holds the parameter layout) --------------------------------
 constexpr int kCh[5] = {1, 32, 64, 128, 128};
@@ -61,41 +61,36 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 // ---- operand loaders -------------------------------------------------------------------------------
 // K-major loaders return the address of the 8 reduction elements [k, k + 8) of operand row `row`;
 // MN-major loaders the address of the 8 row elements [mn, mn + 8) at reduction index k; nullptr where
-// the operand is zero.  kdim(K) is the reduction length of the CTA's GEMM.
+// the operand is zero.
 
 struct PlainK {  // X[row][k] = p[row * ld + k]
   const bf16* p;
   int ld, rows;
   __device__ const bf16* kchunk(int row, int k) const { return row < rows ? p + (size_t)row * ld + k : nullptr; }
-  __device__ int kdim(int K) const { return K; }
-  __device__ int zsplit() const { return blockIdx.z; }
 };
 
 struct PlainMN {  // X[mn][k] = p[k * ld + mn]
   const bf16* p;
   int ld, cols;
   __device__ const bf16* mnchunk(int mn, int k) const { return mn < cols ? p + (size_t)k * ld + mn : nullptr; }
-  __device__ int kdim(int K) const { return K; }
-  __device__ int zsplit() const { return blockIdx.z; }
 };
 
 // ---- epilogues ---------------------------------------------------------------------------------------
-// apply(row, col0, v[16], acc): the accumulator's row `row`, columns [col0, col0 + 16) of the CTA's tile
-// (global indices); acc is a per-thread running value; finish(...) runs once per thread after all
-// columns, with the CTA's shared scratch (all threads call it).
+// apply(row, col0, v[16], scratch): the accumulator's row `row`, columns [col0, col0 + 16) of the CTA's tile
+// (global indices); finish(scratch, ...) runs once per thread after all columns (all threads call it).
 
 // FP32 rows of split z: part[z * zstride + row * ld + col].
 struct EpiF32 {
   float* part;
   long long zstride;
   int rows, ld;
-  __device__ void apply(int row, int col0, float v[16], float&, float*) const {
+  __device__ void apply(int row, int col0, float v[16], float*) const {
     if (row >= rows) return;
     float4* d = reinterpret_cast<float4*>(part + blockIdx.z * zstride + (size_t)row * ld + col0);
 #pragma unroll
     for (int q = 0; q < 4; ++q) d[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
   }
-  __device__ void finish(int, float, float*, int, int, int) const {}
+  __device__ void finish(float*, int, int, int) const {}
 };
 
 // Transposed FP32 store of split z: out[z * zstride + col * ld + row] for row < rows (coalesced: the
@@ -104,13 +99,13 @@ struct EpiF32T {
   float* out;
   long long zstride;
   int rows, ld;
-  __device__ void apply(int row, int col0, float v[16], float&, float*) const {
+  __device__ void apply(int row, int col0, float v[16], float*) const {
     if (row >= rows) return;
     float* d = out + blockIdx.z * zstride + (size_t)col0 * ld + row;
 #pragma unroll
     for (int j = 0; j < 16; ++j) d[(size_t)j * ld] = v[j];
   }
-  __device__ void finish(int, float, float*, int, int, int) const {}
+  __device__ void finish(float*, int, int, int) const {}
 };
 
 // Sum 16 per-lane values over the warp's 32 lanes by recursive halving (16 shuffles); lane l ends with
@@ -141,7 +136,7 @@ struct EpiDfeat {
   const bf16* feat;  // [B][kFeatPitch]
   float* colpart;
   int nb;
-  __device__ void apply(int row, int col0, float v[16], float&, float* scratch) const {
+  __device__ void apply(int row, int col0, float v[16], float* scratch) const {
     if (row < nb) {
       const uint4* a = reinterpret_cast<const uint4*>(feat + (size_t)row * kFeatPitch + col0);
       float m[16];
@@ -163,7 +158,7 @@ struct EpiDfeat {
     const float s = warp_sum16(v, lane);
     if ((lane & 1) == 0) scratch[warp * 128 + col0 - blockIdx.y * 128 + sum16_col(lane)] = s;
   }
-  __device__ void finish(int, float, float* scratch, int tid, int mt, int n_mt) const {
+  __device__ void finish(float* scratch, int tid, int mt, int n_mt) const {
     __syncthreads();
     if (tid < 128) {
       const float s = scratch[tid] + scratch[128 + tid] + scratch[256 + tid] + scratch[384 + tid];
@@ -173,14 +168,14 @@ struct EpiDfeat {
 };
 
 // ---- the GEMM kernel -------------------------------------------------------------------------------
-// S stages of (A, B) slices: 4 for long reductions, fewer where a CTA has only a few slices, so that
-// more CTAs share an SM (at most five: 5 x 32 ... 2 x 128 tensor-memory columns stay within the 512).
-template <int BN, int S>
+// S stages of (A, B) slices: 4 for long reductions, fewer where a CTA has only a few slices, so that more CTAs share
+// an SM (three with two stages: 384 of the 512 tensor-memory columns).
+template <int S>
 struct Cfg {
   static constexpr int kA = kBM * kBK * 2;  // bytes of one A slice (16 KB)
-  static constexpr int kB = BN * kBK * 2;
+  static constexpr int kB = kBN * kBK * 2;
   static constexpr int kStage = kA + kB;
-  static constexpr int kScratch = 4 * BN * 4;  // epilogue column sums [warp][BN]
+  static constexpr int kScratch = 4 * kBN * 4;  // epilogue column sums [warp][kBN]
   static constexpr size_t kSmem = 1024 + (size_t)S * kStage + 128 + kScratch;
 };
 
@@ -217,38 +212,35 @@ __device__ __forceinline__ uint64_t slice_desc(uint32_t a, int j) {
   return tc::smem_desc(a + j * 2 * (ROWS / 8) * 128, (ROWS / 8) * 128, 128);
 }
 
-// C tiles (128 x BN) of rows [mt 128, mt 128 + 128) for mt = blockIdx.x, blockIdx.x + gridDim.x, ...
-// (n_mt row tiles in all), columns from blockIdx.y BN; blockIdx.z = split of the reduction (kchunk
-// each) or, for the data gradient, the parity class (its loaders read blockIdx.z).  The tensor memory
-// and the mbarrier ring stay with the CTA across its tiles; g counts the slices issued so far, which
+// C tiles (128 x 128) of rows [mt 128, mt 128 + 128) for mt = blockIdx.x, blockIdx.x + gridDim.x, ...
+// (n_mt row tiles in all), columns from blockIdx.y 128; blockIdx.z = split of the reduction (kchunk each).  The
+// tensor memory and the mbarrier ring stay with the CTA across its tiles; g counts the slices issued so far, which
 // selects the stage buffer (g mod S) and the mbarrier phase (g div S).
-template <int BN, int kStages, bool AMN, bool BMN, class LA, class LB, class EP>
-__global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2 ? 4 : (kStages == 3 ? 3 : 2)) : 1)) k_cnn_gemm(const LA la, const LB lb, const EP ep, int n_mt, int K, int kchunk,
+template <int kStages, bool AMN, bool BMN, class LA, class LB, class EP>
+__global__ void __launch_bounds__(kThr, 1) k_cnn_gemm(const LA la, const LB lb, const EP ep, int n_mt, int K, int kchunk,
                                                       unsigned* status, unsigned wait_limit, const void* any) {
-  using C = Cfg<BN, kStages>;
+  using C = Cfg<kStages>;
   extern __shared__ unsigned char smem_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bar = (uint64_t*)(sm + kStages * C::kStage);
   uint32_t* tslot = (uint32_t*)(bar + kStages);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.y * BN;
-  const int Kz = la.kdim(K);
-  const long long kb0 = (long long)la.zsplit() * kchunk;
-  const int kb = kb0 >= Kz ? Kz : (int)kb0;
-  const int ke = (int)min((long long)Kz, (long long)kb + kchunk);
+  const int n0 = blockIdx.y * kBN;
+  const int kb = (int)min((long long)K, (long long)blockIdx.z * kchunk);
+  const int ke = (int)min((long long)K, (long long)kb + kchunk);
   const int nk = ke > kb ? (ke - kb + kBK - 1) / kBK : 0;
   if (tid == 0) {
 #pragma unroll
     for (int s = 0; s < kStages; ++s) tc::mbar_init(bar + s, 1);
     tc::mbar_init_fence();
   }
-  if (warp == 0) tc::tmem_alloc(tslot, BN);
+  if (warp == 0) tc::tmem_alloc(tslot, kBN);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *tslot;
   const uint32_t sbase = tc::smem_u32(sm);
-  constexpr uint32_t idesc = tc::idesc_bf16(kBM, BN, AMN, BMN);
+  constexpr uint32_t idesc = tc::idesc_bf16(kBM, kBN, AMN, BMN);
   float* scratch = reinterpret_cast<float*>((uint8_t*)bar + 128);  // the epilogue's column sums
   int ok = 1;
   unsigned g = 0;
@@ -259,7 +251,7 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
       if (s < nk) {
         const uint32_t sa = sbase + ((g + s) % kStages) * C::kStage;
         fill<kBM, AMN>(la, sa, m0, kb + s * kBK, ke, any);
-        fill<BN, BMN>(lb, sa + C::kA, n0, kb + s * kBK, ke, any);
+        fill<kBN, BMN>(lb, sa + C::kA, n0, kb + s * kBK, ke, any);
       }
       cp_commit();
     }
@@ -280,7 +272,7 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
         const uint32_t sa = sbase + (gc % kStages) * C::kStage, sb = sa + C::kA;
 #pragma unroll
         for (int j = 0; j < kBK / 16; ++j)
-          tc::mma_bf16(tmem, slice_desc<kBM, AMN>(sa, j), slice_desc<BN, BMN>(sb, j), idesc, (c > 0 || j > 0) ? 1u : 0u);
+          tc::mma_bf16(tmem, slice_desc<kBM, AMN>(sa, j), slice_desc<kBN, BMN>(sb, j), idesc, (c > 0 || j > 0) ? 1u : 0u);
         tc::mma_commit(bar + gc % kStages);
       }
       issued = c + 1;
@@ -290,7 +282,7 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
         if (ok) {
           const uint32_t sa = sbase + ((g + nxt) % kStages) * C::kStage;
           fill<kBM, AMN>(la, sa, m0, kb + nxt * kBK, ke, any);
-          fill<BN, BMN>(lb, sa + C::kA, n0, kb + nxt * kBK, ke, any);
+          fill<kBN, BMN>(lb, sa + C::kA, n0, kb + nxt * kBK, ke, any);
         }
       }
       cp_commit();
@@ -305,19 +297,18 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
     // the next tile's first copies go out now, so that they land while this tile's epilogue runs
     const int next = mt + gridDim.x;
     if (next < n_mt) prologue(next * kBM);
-    float acc = 0.f;
     const int row = m0 + warp * 32 + lane;
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
+    for (int c0 = 0; c0 < kBN; c0 += 16) {
       float v[16];
       tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
       if (issued == 0) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = 0.f;
       }
-      ep.apply(row, n0 + c0, v, acc, scratch);
+      ep.apply(row, n0 + c0, v, scratch);
     }
-    ep.finish(row, acc, scratch, tid, mt, n_mt);
+    ep.finish(scratch, tid, mt, n_mt);
     // the accumulator and the scratch are free again before the next tile's MMAs
     tc::fence_before();
     __syncthreads();
@@ -328,12 +319,11 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
   if (!ok) {  // the same for the whole CTA
     for (; mt < n_mt; mt += gridDim.x)
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
+      for (int c0 = 0; c0 < kBN; c0 += 16) {
         float v[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = __int_as_float(0x7fffffff);
-        float acc = 0.f;
-        ep.apply(mt * kBM + warp * 32 + lane, n0 + c0, v, acc, scratch);
+        ep.apply(mt * kBM + warp * 32 + lane, n0 + c0, v, scratch);
       }
     if (tid == 0) atomicExch(status, 1u);
   }
@@ -341,7 +331,7 @@ __global__ void __launch_bounds__(kThr, BN == 32 ? 5 : (BN == 64 ? (kStages == 2
   __syncthreads();
   if (warp == 0) {
     tc::fence_after();
-    tc::tmem_dealloc(tmem, BN);
+    tc::tmem_dealloc(tmem, kBN);
   }
 }
 
@@ -680,12 +670,12 @@ __global__ void k_feat_tail(bf16* __restrict__ feat, const float* __restrict__ c
 
 unsigned grid_of(long long n) { return (unsigned)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152LL * 16)); }
 
-// One GEMM launch: M rows of C in 128-row tiles, gy column tiles of BN, gz splits (or classes).
-template <int BN, int S, bool AMN, bool BMN, class LA, class LB, class EP>
+// One GEMM launch: M rows of C in 128-row tiles, gy column tiles, gz splits.
+template <int S, bool AMN, bool BMN, class LA, class LB, class EP>
 cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy, int gz, int kchunk, const void* any,
                  unsigned* status, cudaStream_t st) {
-  using C = Cfg<BN, S>;
-  auto kern = k_cnn_gemm<BN, S, AMN, BMN, LA, LB, EP>;
+  using C = Cfg<S>;
+  auto kern = k_cnn_gemm<S, AMN, BMN, LA, LB, EP>;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmem);
@@ -696,7 +686,7 @@ cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int K, int gy,
   // row tiles per CTA: enough CTAs for every SM to hold as many as its shared memory allows, several
   // tiles each when there are more
   const int n_mt = (M + kBM - 1) / kBM;
-  const long long per_sm = std::max(1, std::min(5, (int)(227 * 1024 / C::kSmem)));
+  const long long per_sm = std::max(1, std::min(512 / kBN, (int)(227 * 1024 / C::kSmem)));
   const long long total = (long long)n_mt * gy * gz, target = 4LL * 152 * per_sm;
   const int per_cta = (int)std::max(1LL, (total + target - 1) / target);
   const int gx = (n_mt + per_cta - 1) / per_cta;
@@ -808,7 +798,7 @@ cudaError_t cnn_tc_forward(const CnnNet& net, const float* img, const float* cs,
   // dense layer: K = 8200 split 16 ways into FP32 partials, then summed with bias and ReLU
   const int Z = 16, kc = chunk_of(kFeatPitch, Z);
   const EpiF32 ep{t.part, (long long)B * kHid, B, kHid};
-  TC_TRY((gemm<128, 4, false, false>(PlainK{(const bf16*)t.feat, kFeatPitch, B}, PlainK{(const bf16*)t.w1b, kFeatPitch, kHid},
+  TC_TRY((gemm<4, false, false>(PlainK{(const bf16*)t.feat, kFeatPitch, B}, PlainK{(const bf16*)t.w1b, kFeatPitch, kHid},
                                   ep, B, kFeatPitch, 1, Z, kc, any, t.status, st)));
   k_sum_z<<<(unsigned)(((long long)B * kHid + 31) / 32), 256, 0, st>>>(t.part, Z, (long long)B * kHid, net.b1, kHid, h, t.status);
   note_launches(1);
@@ -821,12 +811,12 @@ cudaError_t cnn_tc_backward(int B, const CnnTc& t, const float* dh, const CnnGra
   const cudaError_t ez = cudaMemsetAsync(t.tickets, 0, kColTickets * sizeof(unsigned), st);
   if (ez != cudaSuccess) return ez;
   // dense layer: dW1[n][f] = sum_b dh[b][n] feat[b][f] (rows f, both operands MN-major)
-  TC_TRY((gemm<128, 3, true, true>(PlainMN{(const bf16*)t.feat, kFeatPitch, kFeatPitch}, PlainMN{(const bf16*)t.dhb, kHid, kHid},
+  TC_TRY((gemm<3, true, true>(PlainMN{(const bf16*)t.feat, kFeatPitch, kFeatPitch}, PlainMN{(const bf16*)t.dhb, kHid, kHid},
                                 EpiF32T{g.w1, 0, kFeat + 2, kFeat + 2}, kFeatPitch, B, 1, 1, B, any, t.status, st)));
   // ... and dfeat[b][f] = sum_n dh[b][n] W1[n][f] (rows b, B MN-major) -> dY of the last convolution
   // (masked, BF16) and its per-channel column sums
   const int nmt = (B + kBM - 1) / kBM;
-  TC_TRY((gemm<128, 2, false, true>(PlainK{(const bf16*)t.dhb, kHid, B}, PlainMN{(const bf16*)t.w1b, kFeatPitch, kFeat},
+  TC_TRY((gemm<2, false, true>(PlainK{(const bf16*)t.dhb, kHid, B}, PlainMN{(const bf16*)t.w1b, kFeatPitch, kFeat},
                                     EpiDfeat{(bf16*)t.dy3, (const bf16*)t.feat, t.colpart, B}, B, kHid, kFeat / 128, 1,
                                     kHid, any, t.status, st)));
   TC_TRY(colreduce(t.colpart, (kFeat / 128) * nmt, 128, 128, g.b[3], t.part, t.tickets, t.status, st));
