@@ -115,7 +115,7 @@ digs_status digs_count_pairs(const DigsGaussians* g, const DigsLattice* lat, con
 
 /* Forward projection: deform the Gaussians at each projection's weights (Eq. 7-11) and integrate them
  * along every detector ray (Eq. 1, 3, 4), writing proj[P][nv][nu].  All views in one call must share
- * nu and nv.  views: host array [P]. */
+ * nu and nv; a projection is the same, bit for bit, whichever views are beside it.  views: host array [P]. */
 digs_status digs_project_fwd(const DigsGaussians* g, const DigsLattice* lat, const float* phi, const float* w,
                              const DigsView* views, int P, const DigsOpts* opts, float* proj,
                              void* ws, size_t ws_bytes, void* stream);

@@ -20,17 +20,17 @@
 // for them, its share of the pixels one 64-pixel box after another.
 //
 // What bounds them: the latency of a tile's chain of copies, MMAs and epilogue with one tile after another on an SM; at
-// batch 256 HBM runs at 15 to 36 % of its peak, the L2 at 15 to 22 % and the tensor pipe at 14 to 30 %.  (Keeping
-// layer 1's weights in shared memory, a third of its fill, changed nothing: 411 and 406 us a training step.)
+// batch 256 HBM runs at 15 to 48 % of its peak, the L2 at 15 to 35 % and the tensor pipe at 13 to 39 %.  (Keeping
+// layer 1's weights in shared memory, a third of its fill, changed nothing.)
 // The form before this one gathered 16 bytes per thread and cp.async, with the address arithmetic of a tap for
 // each, on the threads that also ran the epilogue, and stored 16 bytes per lane at a distance of 128.
-// Launch times at batch 256, layers 1 / 2 / 3, before and now: forward 97 / 62 / 39 -> 32 / 19 / 12 us, data
-// gradient 167 / 102 / 51 -> 33 / 28 / 18, weight gradient 103 / 67 / 35 -> 23 / 17 / 13; the training step
-// 978 -> 443 us, inference of 680 projections 745 -> 378 us.  The multiply-adds of every output element are added in
-// the same order as before.
+// Launch times at batch 256, layers 1 / 2 / 3, before and now: forward 97 / 62 / 39 -> 29 / 18 / 12 us, data
+// gradient 167 / 102 / 51 -> 34 / 28 / 18, weight gradient 103 / 67 / 35 -> 29 / 18 / 13; the training step, with the
+// first layer's kernels, 978 -> 418 us, inference of 680 projections 745 -> 346 us.  The multiply-adds of every output
+// element are added in the same order as before.
 // One warp issues the copies, one the MMAs, four run the epilogue on the other half of the tensor memory; CTAs are
-// persistent, one per SM (layer 1's forward two: 411 -> 401 us a training step, 353 -> 343 the inference).  Every wait is bounded: a role that gives up sets *status, waits for what it has in
-// flight and leaves; the sums that follow are NaN (k_sum_z, k_colreduce_once).
+// persistent, one per SM (layer 1's forward two, 2.5 % of a training step).  Every wait is bounded: a role that gives
+// up sets *status, waits for what it has in flight and leaves; the sums that follow are NaN (k_sum_z, k_colreduce_once).
 #include <cuda.h>
 #include <cuda_bf16.h>
 

@@ -33,7 +33,7 @@ struct Workspace {
   uint32_t* seg;          // [2P + 2] each projection's first pair and first sort block
   uint2* ranges;          // [P * T] sorted-range of each (projection, tile)
   uint32_t* order;        // [P * T] forward launch order (longest lists first)
-  float4* grec;           // [P * n * 3] backward: the twelve pixel moments of each (projection, Gaussian) record
+  float4* grec;           // [P * n * 3] backward: the twelve pixel sums of each (projection, Gaussian) record
   uint8_t* bcost;         // [P * n] backward sweep cost of each record: box pixels / 32, capped at 255 (0: culled)
   float* gw_part;         // [pair-sum CTAs][P][R] dL/dw partial sums
   float* ffd;             // [12 R][n_total]: u_r (3R components) then grad u_r (9R) at each mean

@@ -12,23 +12,23 @@
 // 32 records at a time, one per lane, writes an entry for every block whose pixels the record's cutoff ellipse
 // can reach, and sweeps each block's entries, four per step, in list order: no canvas, no atomics, sums that do
 // not depend on timing.  CTAs start in order of decreasing list length.
-// What bounds it: instruction issue, about 25 instructions per entry and block of 64 pixels (FMA and SFU pipes
-// each about 60 % busy), then loading and testing the records.  One block per warp made every block load and
+// What bounds it: instruction issue (69 % of cycles), about 26 instructions per entry and block of 64 pixels (FMA pipe
+// 61 % busy, SFU 38 %), then loading and testing the records.  One block per warp made every block load and
 // test the whole list by itself: a third of the time.  128 thorax projections (100k Gaussians, 256^2):
-// 5.31 -> 4.22 ms; 16: 0.78 -> 0.57; 8 of 500k Gaussians on 512^2: 5.2 -> 3.8; 16 of 2,000 on 64^2:
-// 0.044 -> 0.023.
+// 5.37 -> 4.70 ms; 16: 0.79 -> 0.60; 8 of 500k Gaussians on 512^2: 5.0 -> 4.1; 16 of 2,000 on 64^2:
+// 0.045 -> 0.023.
 //
 // Backward: needs no tile lists.  One half-warp per (projection, Gaussian) record (the two records of a warp of
 // similar box size) sweeps the record's pixel box in 16-column slices, reading g = dL/dI * |X - s| from the
 // projection-sized image (L1/L2 resident).  Narrow slices (w <= 8): lane l owns column (l mod w), starts at row
 // (l div w) and takes the row pair (r, r + s), s = 16 div w, stepping 2s rows; wider slices: the column pair
-// (c, c + ceil(w/2)) of row (l div ceil(w/2)), stepping s = 16 div ceil(w/2) rows.  Each lane accumulates six
-// moments per pixel of its pair; a slice adds their twelve (dx, dy)-moments, the half-warp reduces those with a
-// 12-shuffle recursive halving and twelve lanes write them to the record's slot (no atomics).
-// What bounds it: the FMA pipe (packed arithmetic takes two of its cycles; 70 % busy) and the instructions per
+// (c, c + ceil(w/2)) of row (l div ceil(w/2)), stepping s = 16 div ceil(w/2) rows.  Each lane accumulates the value
+// and six moments per pixel of its pair; a slice adds them to twelve (dx, dy)-moments, the half-warp reduces those with
+// a 12-shuffle recursive halving and twelve lanes write them to the record's slot (no atomics).
+// What bounds it: the FMA pipe (packed arithmetic takes two of its cycles; 65 % busy) and the instructions per
 // record around the sweep (a third of the time).  128 thorax projections (100k Gaussians, 256^2), with the
-// ranking of the records: 8.82 -> 7.36 ms; 16 of 2,000 on 64^2: 0.032 -> 0.027; 64 of four scans of 30k to 200k,
-// whose missing records are no longer visited: 4.9 -> 3.8.
+// ranking of the records: 8.81 -> 7.67 ms; 16 of 2,000 on 64^2: 0.035 -> 0.029; 64 of four scans of 30k to 200k,
+// whose missing records are no longer visited: 5.17 -> 3.97.
 //
 // Loss: per-warp partials of the squared residuals from the forward, summed in two fixed-order levels.
 #include <algorithm>
@@ -512,8 +512,8 @@ __device__ __forceinline__ void group_reduce_store12(const float v[12], float* o
 // against 7.5 ms for 128 thorax projections); where that leaves too few warps, a quarter of the group each (and
 // each quarter's warp ranks the group again, about 45 instructions).
 // The next rounds' records are copied to shared memory by cp.async (double buffer) while one is swept.
-// 28 warps of 72 registers per SM: with 64 registers (32 warps) the loop spills and recomputes its lane layout,
-// with 80 (24 warps) its latencies show (8.05, 7.8 and 9.4 ms with four-warp CTAs).
+// 28 warps of 72 registers per SM (25 of 80: the same); with 64 registers (32 warps) the loop spills and recomputes
+// its lane layout.
 // counts.n[b]: records of projection b that exist (its scan's Gaussians); N: record stride of a projection.
 // Grid: (ceil(warps / W), P), warps = ceil(N / 32) * 32 / (WR * (32 / LPR)).
 struct ViewCounts {
@@ -651,7 +651,7 @@ cudaError_t launch_raster_bwd(const Workspace& ws, const ScanTable& sc, const Vi
       ws.rec, ws.bcost, counts, ws.n, ws.nu, ws.nv, ws.dldi, c2, (float*)ws.grec)
   // A warp per group of 32 records from 8192 groups on, four below: 1000 groups 0.037 / 0.027 ms, 7300 0.117 / 0.111,
   // 12500 0.260 / 0.258, 50000 0.949 / 0.987, 400000 7.36 / 7.79.  One record per warp (32 lanes): always four
-  // warps per group (1000 groups 0.043 / 0.031, 50000 1.28 / 1.16).
+  // warps per group (1000 groups 0.043 / 0.031, 50000 1.28 / 1.16).  (Taken without the sum of g V, which adds 3 % to each.)
   if (ws.bwd_lanes == 32) DIGS_BWD(32, 8, 4);
   else if ((long long)G * ws.P > 8192) DIGS_BWD(16, 16, 1);
   else DIGS_BWD(16, 4, 4);
